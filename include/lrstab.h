@@ -556,14 +556,10 @@ lrs_status lrs_alu_probe(int32_t device, int64_t iters, double* ops_per_s);
  *   LRS_TUNE_AMP_BLOCKS_PER_SM    amplitude grid target, blocks per SM (1..64, 8)
  *   LRS_TUNE_NORM_MAX_TILES       norm estimate, maximum term tiles (1..2^20, 2048)
  *   LRS_TUNE_MC_CHAINS_PER_BLOCK  Metropolis chains per block (1..64, 64)
- *   LRS_TUNE_NORM_MAX_FOLDS       norm estimate: a term with n - |v| <= this
- *                                 value (-1..12, 12) evaluates its exponential
- *                                 sum over y = G x, i.e. the form y^T (A+J) y
- *                                 plus 2 (F s + (A+J) G s) . y restricted to the
- *                                 n - |v| constraints (F^T y)_k = 0, k not in v,
- *                                 instead of forming K = G^T (A+J) G; -1 forms
- *                                 K for every term.  Both give the same exact
- *                                 per-term value.
+ *   LRS_TUNE_NORM_MAX_FOLDS       norm estimate (-1..12, 12): accepted and returned;
+ *                                 every term sums over y = G (s + x) restricted to the
+ *                                 n - |v| constraints, on the route that its |v|
+ *                                 decides, so the value changes nothing.
  *   LRS_TUNE_MC_STAGES            Metropolis: chains whose inputs a block keeps
  *                                 in flight in shared memory (1..4, 1; 12 KB each
  *                                 for one step per pass, 20 KB for two: one stage
@@ -575,11 +571,8 @@ lrs_status lrs_alu_probe(int32_t device, int64_t iters, double* ops_per_s);
  *                                 repeating the per-gate scalar work in every lane;
  *                                 results are bit-identical for every value.
  *                                 Narrower tableaux take one lane per term.
- *   LRS_TUNE_NORM_FUSE_FOLDS      norm estimate: a term that takes the y = G x
- *                                 route with n - |v| <= this value (0..8, 8) folds
- *                                 its constraints into the rows of A+J while the
- *                                 rows are formed (one pass), above it one pass
- *                                 per constraint.  Same exact per-term value.
+ *   LRS_TUNE_NORM_FUSE_FOLDS      norm estimate (0..8, 8): accepted and returned, as
+ *                                 LRS_TUNE_NORM_MAX_FOLDS; changes nothing.
  *   LRS_TUNE_MC_LOOKAHEAD         Metropolis flip chains: steps per pass over the
  *                                 chains' Pauli states (1 or 2, default 2).  With 2
  *                                 one pass forms <y|psi> for step t's proposal and
