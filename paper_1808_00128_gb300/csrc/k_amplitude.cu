@@ -20,37 +20,29 @@
 namespace {
 
 constexpr int AMP_XT = 128;   // threads per block
-// strings per thread (independent chains for ILP): eight for the plain batch (each
-// term's tables and barrier serve 1024 strings), four for the chain start (its
-// per-string state buffers)
-__host__ __device__ constexpr int amp_xp(bool qout) { return qout ? 4 : 8; }
-__host__ __device__ constexpr int amp_xb(bool qout) { return AMP_XT * amp_xp(qout); }
+// strings per thread (independent chains for ILP): each term's tables and barrier
+// serve 1024 strings
+constexpr int AMP_XP = 8, AMP_XB = AMP_XT * AMP_XP;
 
 struct AmpEntry {
     uint64_t u, w, z;
 };
 
-// QOUT: also store every (x_i, term) Pauli state at entry i * cap + alpha of Qout
-// (q_store: 12 bytes for n <= 40, i.e. NCH <= 10, else 16), zero terms included (the
-// Metropolis chain state of Sec. 4.2).
 // PK (n <= 62): only parity(z) enters mu, and parity(z_after) = parity(z) +
 // parity(w & u_q) + parity(z_q), so a table entry keeps parity(z_q) in bit 63 of u_q
 // and the lookups XOR-accumulate w & u_q (one popcount per string at the end): two
 // 8-byte tables (u_q, w_q) instead of three, each a conflict-free 128-byte row per
 // chunk.
-// Register budget: five blocks per SM (96 registers, eight strings per thread) for the
-// plain amplitude batch, six (80 registers, four strings) for the variant that also
-// writes the Pauli states.
-constexpr int amp_min_blocks(bool qout) { return qout ? 6 : 5; }
+// Register budget: five blocks per SM (96 registers, eight strings per thread).
 // ERR: also sum |b_alpha <x|phi_alpha>| over the terms that contribute at x (one FP32
 // add per contributing (x, term)), written to magp[i * n_tiles + tile]: the input of
 // the per-result error bound of k_amp_reduce.
 // One block of the amplitude launch: term tile `tile`, strings xblk * AMP_XB ... (shared
 // by the single-circuit kernel and the batched kernel of several circuits).
-template <int NCH, bool QOUT, bool PK, bool ERR>
+template <int NCH, bool PK, bool ERR>
 __device__ __forceinline__ void amp_block(const TermsView& T, const uint64_t* __restrict__ xs, int64_t batch,
                                           int64_t tt, float2* __restrict__ partial, int64_t n_tiles,
-                                          void* __restrict__ Qout, float* __restrict__ magp, int64_t tile,
+                                          float* __restrict__ magp, int64_t tile,
                                           int64_t xblk) {
     // One barrier per term: while the block evaluates term a from table slot a, it
     // builds the table of term a + 1 (from the rows stored in the previous interval)
@@ -63,18 +55,6 @@ __device__ __forceinline__ void amp_block(const TermsView& T, const uint64_t* __
     __shared__ float val_abs[3];            // |b| 2^{-(|v|+h)/2} (ERR)
     __shared__ uint64_t sc[3][4];           // glo, ghi, v, s
     __shared__ uint32_t sc_live[3];
-    // compact Pauli states of the last QG terms for each of the block's strings, private
-    // to the thread that owns the string: written out as 16-byte vectors every QG terms
-    constexpr int AMP_XP = amp_xp(QOUT), AMP_XB = amp_xb(QOUT);
-    constexpr bool CQ = QOUT && NCH <= 10;
-    constexpr int QG = 4;
-    __shared__ uint64_t qb8[CQ ? QG : 1][CQ ? AMP_XB : 1];
-    __shared__ uint32_t qb4[CQ ? QG : 1][CQ ? AMP_XB : 1];
-    // the 16-byte states (n > 40) of the last QW terms, written out as one full 32-byte
-    // sector per string every QW terms (a store per term would write half sectors)
-    constexpr bool WQ = QOUT && !CQ;
-    constexpr int QW = 2;
-    __shared__ uint64_t qwu[WQ ? QW : 1][WQ ? AMP_XB : 1], qww[WQ ? QW : 1][WQ ? AMP_XB : 1];
     const int n = T.n;
     const int tid = threadIdx.x;
     const int64_t xb = xblk * AMP_XB;
@@ -165,7 +145,7 @@ __device__ __forceinline__ void amp_block(const TermsView& T, const uint64_t* __
         if (a + 2 < a1) store(tb, (kt + 2) % 3);
         if (a + 3 < a1) prefetch(a + 3);
         const bool live = sc_live[ss] != 0u;
-        if (QOUT || live) {
+        if (live) {
             const uint64_t glo = sc[ss][0], ghi = sc[ss][1], v = sc[ss][2], s = sc[ss][3];
             const uint64_t nv = ~v & T.nmask, sv = s & v;
     #pragma unroll
@@ -199,53 +179,13 @@ __device__ __forceinline__ void amp_block(const TermsView& T, const uint64_t* __
                     zpar = par64(z);
                 }
                 const int mu = __popcll(x & glo) + 2 * __popcll(x & ghi) + 2 * (int)zpar;
-                if (CQ) {
-                    const int g = (int)((a - a0) & (QG - 1));
-                    qb8[g][tid + k * AMP_XT] = u | (w << 40);
-                    qb4[g][tid + k * AMP_XT] = (uint32_t)(w >> 24) | ((uint32_t)(mu & 3) << 16);
-                } else if (WQ) {
-                    const int g = (int)((a - a0) & (QW - 1));
-                    qwu[g][tid + k * AMP_XT] = u | ((uint64_t)(mu & 3) << 62);   // the q_store layout
-                    qww[g][tid + k * AMP_XT] = w;
-                }
-                if (live && ((u ^ s) & nv) == 0) {
+                if (((u ^ s) & nv) == 0) {
                     const int sign = (int)par64(u & (w ^ sv));
                     acc[k].add(val8[ss][(2 * mu + 4 * sign) & 7]);
                     if (ERR) mag[k] += val_abs[ss];
                 }
             }
-            if (CQ && ((a - a0) & (QG - 1)) == QG - 1) {
-                // terms a-3 .. a of each of the thread's strings: 32 bytes of u | w << 40 and
-                // 16 bytes of (w >> 24) | mu << 16, contiguous and 16-byte aligned (a0 and
-                // the tile length are multiples of QG, cap of 256)
-                uint64_t* q8 = reinterpret_cast<uint64_t*>(Qout);
-                uint32_t* q4 = reinterpret_cast<uint32_t*>(q8 + batch * T.cap);
-    #pragma unroll
-                for (int k = 0; k < AMP_XP; ++k) {
-                    const int sl = tid + k * AMP_XT;
-                    const int64_t i = xb + sl;
-                    if (i >= batch) continue;
-                    const int64_t e = i * T.cap + a - (QG - 1);
-                    reinterpret_cast<ulonglong2*>(q8 + e)[0] = make_ulonglong2(qb8[0][sl], qb8[1][sl]);
-                    reinterpret_cast<ulonglong2*>(q8 + e)[1] = make_ulonglong2(qb8[2][sl], qb8[3][sl]);
-                    *reinterpret_cast<uint4*>(q4 + e) = make_uint4(qb4[0][sl], qb4[1][sl], qb4[2][sl], qb4[3][sl]);
-                }
-            }
-            if (WQ && ((a - a0) & (QW - 1)) == QW - 1) {
-                // terms a-1, a of each of the thread's strings: one 32-byte sector (a0
-                // and the tile length are even, cap a multiple of 256)
-                ulonglong2* q16 = reinterpret_cast<ulonglong2*>(Qout);
-#pragma unroll
-                for (int k = 0; k < AMP_XP; ++k) {
-                    const int sl = tid + k * AMP_XT;
-                    const int64_t i = xb + sl;
-                    if (i >= batch) continue;
-                    const int64_t e = i * T.cap + a - (QW - 1);
-                    q16[e] = make_ulonglong2(qwu[0][sl], qww[0][sl]);
-                    q16[e + 1] = make_ulonglong2(qwu[1][sl], qww[1][sl]);
-                }
-            }
-        }   // live (every term for the Pauli-state output)
+        }
         __syncthreads();   // slot tb ^ 1 and the next rows and scalars are complete
     }
 #pragma unroll
@@ -258,12 +198,12 @@ __device__ __forceinline__ void amp_block(const TermsView& T, const uint64_t* __
     }
 }
 
-template <int NCH, bool QOUT, bool PK, bool ERR>
-__global__ void __launch_bounds__(AMP_XT, amp_min_blocks(QOUT)) k_amplitude(TermsView T, const uint64_t* __restrict__ xs,
+template <int NCH, bool PK, bool ERR>
+__global__ void __launch_bounds__(AMP_XT, 5) k_amplitude(TermsView T, const uint64_t* __restrict__ xs,
                                                       int64_t batch, int64_t tt,
                                                       float2* __restrict__ partial, int64_t n_tiles,
-                                                      void* __restrict__ Qout, float* __restrict__ magp) {
-    amp_block<NCH, QOUT, PK, ERR>(T, xs, batch, tt, partial, n_tiles, Qout, magp, blockIdx.x, blockIdx.y);
+                                                      float* __restrict__ magp) {
+    amp_block<NCH, PK, ERR>(T, xs, batch, tt, partial, n_tiles, magp, blockIdx.x, blockIdx.y);
 }
 
 // Several circuits of the same width in one launch: block b runs block b - first[c]
@@ -282,15 +222,14 @@ struct AmpBatch {
 };
 
 template <int NCH, bool PK>
-__global__ void __launch_bounds__(AMP_XT, amp_min_blocks(false)) k_amplitude_batch(const __grid_constant__ AmpBatch B) {
+__global__ void __launch_bounds__(AMP_XT, 5) k_amplitude_batch(const __grid_constant__ AmpBatch B) {
     const int64_t b = blockIdx.x;
     int c = 0;
 #pragma unroll 1
     for (int i = 1; i < B.count; ++i)
         if (B.first[i] <= b) c = i;
     const int64_t local = b - B.first[c];
-    amp_block<NCH, false, PK, false>(B.T[c], B.xs[c], B.batch[c], B.tt[c], B.partial[c], B.n_tiles[c], nullptr,
-                                     nullptr, local % B.n_tiles[c], local / B.n_tiles[c]);
+    amp_block<NCH, PK, false>(B.T[c], B.xs[c], B.batch[c], B.tt[c], B.partial[c], B.n_tiles[c], nullptr, local % B.n_tiles[c], local / B.n_tiles[c]);
 }
 
 // FP64 sum of the block partials of each x, and (magp != NULL) the error bound of
@@ -383,9 +322,9 @@ struct AmpPlan {
 };
 
 // Term tiles so that the grid covers every SM several times.
-AmpPlan amp_plan(const lrs_ctx* ctx, int64_t batch, bool qout) {
+AmpPlan amp_plan(const lrs_ctx* ctx, int64_t batch, int per_block) {
     AmpPlan P;
-    P.xblocks = (batch + amp_xb(qout) - 1) / amp_xb(qout);
+    P.xblocks = (batch + per_block - 1) / per_block;
     const int64_t target = (int64_t)ctx->sm_count * ctx->tune_amp_bps;
     int64_t nt = (target + P.xblocks - 1) / P.xblocks;
     const int64_t maxt = (ctx->cap + 31) / 32;
@@ -398,51 +337,44 @@ AmpPlan amp_plan(const lrs_ctx* ctx, int64_t batch, bool qout) {
 
 template <int NCH>
 lrs_status launch_amp_t(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* partial,
-                        const AmpPlan& P, void* Qout, float* magp, cudaStream_t st) {
+                        const AmpPlan& P, float* magp, cudaStream_t st) {
     dim3 grid((unsigned)P.n_tiles, (unsigned)P.xblocks);
     const bool pk = ctx->n <= 62;
     const TermsView T = ctx->view();
-    if (Qout)   // chains need n <= 62 (mu lives in bits 62-63 of Q), so the packed tables apply
-        k_amplitude<NCH, true, true, false><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles, Qout,
-                                                                    nullptr);
-    else if (pk && magp)
-        k_amplitude<NCH, false, true, true><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles,
-                                                                    nullptr, magp);
+    if (pk && magp)
+        k_amplitude<NCH, true, true><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles, magp);
     else if (pk)
-        k_amplitude<NCH, false, true, false><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles,
-                                                                     nullptr, nullptr);
+        k_amplitude<NCH, true, false><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles, nullptr);
     else if (magp)
-        k_amplitude<NCH, false, false, true><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles,
-                                                                     nullptr, magp);
+        k_amplitude<NCH, false, true><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles, magp);
     else
-        k_amplitude<NCH, false, false, false><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles,
-                                                                      nullptr, nullptr);
+        k_amplitude<NCH, false, false><<<grid, AMP_XT, 0, st>>>(T, x, batch, P.tt, partial, P.n_tiles, nullptr);
     LRS_LAUNCH_CHECK("amplitude kernel");
     return LRS_OK;
 }
 
 lrs_status launch_amp_kernels(lrs_ctx* ctx, const uint64_t* x, int64_t batch, double* out,
-                              float2* partial, const AmpPlan& P, cudaStream_t st, void* Qout,
+                              float2* partial, const AmpPlan& P, cudaStream_t st,
                               float* magp = nullptr, float* err = nullptr) {
     if (P.xblocks > 65535) return lrs_fail(LRS_ERR_UNSUPPORTED, "amplitude batch too large");
     lrs_status rc;
     switch ((ctx->n + 3) / 4) {
-        case 1: rc = launch_amp_t<1>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 2: rc = launch_amp_t<2>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 3: rc = launch_amp_t<3>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 4: rc = launch_amp_t<4>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 5: rc = launch_amp_t<5>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 6: rc = launch_amp_t<6>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 7: rc = launch_amp_t<7>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 8: rc = launch_amp_t<8>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 9: rc = launch_amp_t<9>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 10: rc = launch_amp_t<10>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 11: rc = launch_amp_t<11>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 12: rc = launch_amp_t<12>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 13: rc = launch_amp_t<13>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 14: rc = launch_amp_t<14>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        case 15: rc = launch_amp_t<15>(ctx, x, batch, partial, P, Qout, magp, st); break;
-        default: rc = launch_amp_t<16>(ctx, x, batch, partial, P, Qout, magp, st); break;
+        case 1: rc = launch_amp_t<1>(ctx, x, batch, partial, P, magp, st); break;
+        case 2: rc = launch_amp_t<2>(ctx, x, batch, partial, P, magp, st); break;
+        case 3: rc = launch_amp_t<3>(ctx, x, batch, partial, P, magp, st); break;
+        case 4: rc = launch_amp_t<4>(ctx, x, batch, partial, P, magp, st); break;
+        case 5: rc = launch_amp_t<5>(ctx, x, batch, partial, P, magp, st); break;
+        case 6: rc = launch_amp_t<6>(ctx, x, batch, partial, P, magp, st); break;
+        case 7: rc = launch_amp_t<7>(ctx, x, batch, partial, P, magp, st); break;
+        case 8: rc = launch_amp_t<8>(ctx, x, batch, partial, P, magp, st); break;
+        case 9: rc = launch_amp_t<9>(ctx, x, batch, partial, P, magp, st); break;
+        case 10: rc = launch_amp_t<10>(ctx, x, batch, partial, P, magp, st); break;
+        case 11: rc = launch_amp_t<11>(ctx, x, batch, partial, P, magp, st); break;
+        case 12: rc = launch_amp_t<12>(ctx, x, batch, partial, P, magp, st); break;
+        case 13: rc = launch_amp_t<13>(ctx, x, batch, partial, P, magp, st); break;
+        case 14: rc = launch_amp_t<14>(ctx, x, batch, partial, P, magp, st); break;
+        case 15: rc = launch_amp_t<15>(ctx, x, batch, partial, P, magp, st); break;
+        default: rc = launch_amp_t<16>(ctx, x, batch, partial, P, magp, st); break;
     }
     if (rc != LRS_OK) return rc;
     k_amp_reduce<<<(unsigned)batch, 256, 0, st>>>(partial, magp, P.n_tiles, batch, P.tt, out, err);
@@ -452,29 +384,29 @@ lrs_status launch_amp_kernels(lrs_ctx* ctx, const uint64_t* x, int64_t batch, do
 
 }  // namespace
 
-// Amplitudes of x[0..batch) into scratch (*amp_out, 2 doubles per x) and the Pauli
-// state Q[i * cap + alpha] of every (x_i, term): the chain start of Sec. 4.2.
-lrs_status launch_amplitude_q(lrs_ctx* ctx, const uint64_t* x, int64_t batch, void* Q, double** amp_out,
-                              cudaStream_t st) {
-    const AmpPlan P = amp_plan(ctx, batch, true);
+// Amplitudes of the chains' start strings into scratch (*amp_out, 2 doubles per x), on the
+// term tiles of 512 strings per block.
+lrs_status launch_amplitude_start(lrs_ctx* ctx, const uint64_t* x, int64_t batch, double** amp_out, cudaStream_t st) {
+    AmpPlan P = amp_plan(ctx, batch, 512);
+    P.xblocks = (batch + AMP_XB - 1) / AMP_XB;
     const size_t part = ((size_t)batch * P.n_tiles * sizeof(float2) + 255) & ~(size_t)255;
     void* scr = nullptr;
     lrs_status rc = lrs_scratch(ctx, part + (size_t)batch * 2 * sizeof(double), &scr);
     if (rc != LRS_OK) return rc;
     *amp_out = (double*)((char*)scr + part);
-    return launch_amp_kernels(ctx, x, batch, *amp_out, (float2*)scr, P, st, Q);
+    return launch_amp_kernels(ctx, x, batch, *amp_out, (float2*)scr, P, st);
 }
 
 lrs_status launch_amplitude(lrs_ctx* ctx, const uint64_t* x, int64_t batch, double* out, float* err,
                             cudaStream_t st) {
     if (batch == 0) return LRS_OK;
-    const AmpPlan P = amp_plan(ctx, batch, false);
+    const AmpPlan P = amp_plan(ctx, batch, AMP_XB);
     const size_t part = ((size_t)batch * P.n_tiles * sizeof(float2) + 255) & ~(size_t)255;
     void* scr = nullptr;
     lrs_status rc = lrs_scratch(ctx, part + (err ? (size_t)batch * P.n_tiles * sizeof(float) : 0), &scr);
     if (rc != LRS_OK) return rc;
     float* magp = err ? (float*)((char*)scr + part) : nullptr;
-    return launch_amp_kernels(ctx, x, batch, out, (float2*)scr, P, st, nullptr, magp, err);
+    return launch_amp_kernels(ctx, x, batch, out, (float2*)scr, P, st, magp, err);
 }
 
 template <int NCH>
@@ -503,7 +435,7 @@ lrs_status launch_amplitude_batch(lrs_ctx* const* ctxs, const uint64_t* const* x
         for (int32_t i = base; i < end; ++i) {
             if (batch[i] == 0) continue;
             lrs_ctx* c = ctxs[i];
-            const AmpPlan P = amp_plan(c, batch[i], false);
+            const AmpPlan P = amp_plan(c, batch[i], AMP_XB);
             if (P.xblocks > 65535) return lrs_fail(LRS_ERR_UNSUPPORTED, "amplitude batch too large");
             void* scr = nullptr;
             lrs_status rc = lrs_scratch(c, (size_t)batch[i] * P.n_tiles * sizeof(float2), &scr);
@@ -600,11 +532,11 @@ extern "C" lrs_status lrs_amplitude_noalloc(lrs_ctx* ctx, const uint64_t* x, int
     lrs_status rc = noalloc_address(ctx->device, &partial);   // first call on a device: set-up
     if (rc != LRS_OK) return rc;
     if (batch == 0) return LRS_OK;
-    const AmpPlan P = amp_plan(ctx, batch, false);
+    const AmpPlan P = amp_plan(ctx, batch, AMP_XB);
     if ((uint64_t)batch * (uint64_t)P.n_tiles > (uint64_t)LRS_NOALLOC_PARTIALS)
         return lrs_fail(LRS_ERR_ARG,
                         "lrs_amplitude_noalloc: %lld partial sums (batch x term tiles) exceed the "
                         "fixed buffer of %u; use a smaller batch or lrs_amplitude",
                         (long long)(batch * P.n_tiles), LRS_NOALLOC_PARTIALS);
-    return launch_amp_kernels(ctx, x, batch, out, partial, P, (cudaStream_t)stream, nullptr);
+    return launch_amp_kernels(ctx, x, batch, out, partial, P, (cudaStream_t)stream);
 }

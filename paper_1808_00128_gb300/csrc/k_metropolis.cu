@@ -1,43 +1,33 @@
-// Metropolis chains with the incremental Pauli update of Sec. 4.2.
+// Metropolis chains (Sec. 4.2) on bit-planes of the terms.
 //
-// State per (chain c, term alpha): Q = i^mu X(u) Z(w) = U_C^{-1} X(x_c) U_C,
-// packed in 12 bytes for n <= 40 and 16 bytes up to n = 62 (q_store), layout
-// [chain][term].
-// A step proposes y = x ^ e_j; every term updates Q_y = Q_x P_j with
-// P_j = U_C^{-1} X_j U_C = i^{gamma_j} X(F_j) Z(M_j):
-//     mu += gamma_j + 2 parity(w & F_j);  u ^= F_j;  w ^= M_j
-// and contributes b <0|Q_y U_H|s> (Eq. (amplitude1)).  Q is written back only
-// for accepted moves, lazily, at the start of the next step.  The accept test
-// is done in FP64 per chain by a separate small kernel.
+// For one term <x|phi> is b omega 2^{-|v|/2} i^{q(x)} where the constraints F_k . x = s_k (column
+// k of F, k not in v) hold, and zero elsewhere, with the Z4 form
+//     q(x) = sum_p d_p x_p + 2 sum_{p<q} J_pq x_p x_q,   J = M F^T (symmetric),
+//     d_p = gamma_p + 2 F_p . M_p + 2 F_p . (s & v)      (mod 4)
+// (Eqs. (amplitude), (amplitude1) with the Pauli product written out: the sign u . w of
+// U_C^{-1} X(x) U_C = i^mu X(u) Z(w) is the diagonal F_p . M_p because M F^T is symmetric).
+// A proposal y = x ^ e_j changes q by +-d_j + 2 J_j . x and constraint i by its bit at j, so a
+// chain's state is two phase bits and one bit per constraint for every term, and all of it is
+// bitwise over the terms: k_mc_planes stores J, d, the constraints' bits and targets as
+// planes (one bit per term), a thread owns 64 terms (two words) and J_j . x is the XOR of
+// the planes J_jq over the set bits q of x, about n / 2 loads for 64 terms.  The state moves
+// 2 + 2 + (constraints) bits per (chain, term) and pass instead of the 96 or 128 of the
+// Pauli pair (u, w); what is left is the FP32 sum over the terms.
+//
+// Planes are stored with the words of a 256-term tile in the order (w, k): term 128 k + 32 w + l
+// of the tile is bit l of component k of column 4 tile + w.  A thread sums its 64 terms as
+// leaves (k = 0) + (k = 1) and then a binary tree over l, the four columns of a tile in
+// order, the tiles in FP64.
 #include <string.h>
 
 #include "lrs_device.cuh"
 
 namespace {
 
-constexpr int MC_TPB = 128;   // threads per block
-constexpr int MC_TPT = 2;     // terms per thread
-constexpr int MC_TERMS = MC_TPB * MC_TPT;   // terms per block (cap is a multiple of 256)
-constexpr int MC_CG = 64;     // chains per block (grid.y groups)
+constexpr int MC_TPB = 128;    // threads per block
+constexpr int MC_TERMS = 256;  // terms per tile (cap is a multiple of 256)
 
-__device__ __forceinline__ float2 block_sum(float2 v, float2 (*red)[MC_TPB / 32], int slot) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
-    }
-    if ((threadIdx.x & 31) == 0) red[slot][threadIdx.x >> 5] = v;
-    return v;
-}
-
-// b e^{i pi k/4} 2^{-e/2} times i^m (m = mu + 2 sign): the Z8 factor of a term at a
-// string, with the term's part (coefficient, phase k, |v| + h) folded in once.
-__device__ __forceinline__ float2 times_i_pow(float2 z, uint32_t m) {
-    const float2 r = (m & 1u) ? make_float2(-z.y, z.x) : z;
-    return (m & 2u) ? make_float2(-r.x, -r.y) : r;
-}
-
-// ---- bulk-copy pipeline helpers (1-D cp.async.bulk completing on an mbarrier) ----------
+// ---- bulk-copy helpers (1-D cp.async.bulk completing on an mbarrier) ----------
 constexpr unsigned long long MC_WAIT_NS = 1000000000ull;   // 1 s
 __device__ __forceinline__ uint32_t mc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned long long mc_ns() {
@@ -74,373 +64,373 @@ __device__ __forceinline__ bool mc_bar_wait(uint32_t bar, uint32_t parity) {
     return true;
 }
 
-// One chain's inputs for the block's MC_TERMS terms: its Pauli states and the rows
-// F_j, M_j of its proposal and F_p, M_p of its pending accepted flip.
-// At most MC_ST chains in flight per block; the launch takes nst <= MC_ST stages
-// (a tuning knob: two stages, 24 KB, leave room for eight blocks per SM at n = 40,
-// four suit the n = 50 workload).
-constexpr int MC_ST = 4;
-struct McStage {
-    // the chain's Pauli states: MC_TERMS 16-byte pairs, or (compact) MC_TERMS 64-bit
-    // words followed by MC_TERMS 32-bit words
-    __align__(16) unsigned char q[MC_TERMS * 16];
-    uint64_t fj[MC_TERMS], mj[MC_TERMS], fp[MC_TERMS], mp[MC_TERMS];
+// ---- planes -----------------------------------------------------------------------------
+// cols = cap / 64 columns of 64 terms.
+struct McView {
+    int n;
+    int64_t cols;
+    uint2* J;        // [n (n - 1) / 2 + 1][cols]: J_pq, p > q, row p (p - 1) / 2 + q; the last row zero
+    uint2* D;        // [n][2][cols]: d_p, bits 0 and 1
+    uint2* K;        // [n][n][cols]: coefficient of constraint i at qubit p
+    uint2* target;   // [n][cols]: s at constraint i
+    float2* base;    // [64][cols]: b omega 2^{-|v|/2} / 2 of term (k, l), row 32 k + l (0: no contribution)
+    uint8_t* mf;     // [cols / 4]: constraints of the tile (the most of its terms)
 };
+__host__ __device__ __forceinline__ int mc_pairs(int n) { return n * (n - 1) / 2; }
+// Chain states: [plane][chain][cols]: phase bits 0 and 1, the parities J_j1 . x and J_j2 . x of
+// the last pass's proposals, then the constraints' syndromes.
+constexpr int MC_PLANES = 4;
 
-// One proposal: apply the pending accepted flip, then form the amplitude of y.
-// The block owns MC_TERMS consecutive terms; for each of its chains thread 0 copies
-// the 4 KB of Q and the 2 KB row segments (coalesced [row][term] layout) into a
-// shared stage with cp.async.bulk, nst chains ahead, so the HBM stream does not
-// depend on how many loads the threads keep in flight.  Q is written back only
-// where a pending flip is committed.  Each thread owns MC_TPT terms
-// (tid + k * MC_TPB) and sums them before the block reduction.  A stage wait that
-// gives up (1 s) sets *err, stops the block and leaves its partial sums unwritten.
-template <bool CQ>
-__global__ void __launch_bounds__(MC_TPB) k_metro_propose(TermsView T, int64_t C, void* __restrict__ Q,
-                                                          const int32_t* __restrict__ pend,
-                                                          const int32_t* __restrict__ jprop,
-                                                          float2* __restrict__ partial, int64_t n_tiles,
-                                                          int cg, int nst, int* err, int groups_fast) {
-    extern __shared__ __align__(128) unsigned char mc_dyn[];
-    McStage* stage = reinterpret_cast<McStage*>(mc_dyn);
-    __shared__ float2 red[MC_CG][MC_TPB / 32];
-    __shared__ int32_t spj[MC_CG], spq[MC_CG], sj[MC_CG];
-    __shared__ __align__(8) uint64_t full[MC_ST];
-    __shared__ int abort_flag;
-    const int tid = threadIdx.x;
-    // groups_fast: blockIdx.x is the chain group, so the blocks that read the same
-    // term tile's rows F_j, M_j run together and share them through L2
-    const int64_t tile = groups_fast ? blockIdx.y : blockIdx.x;
-    const int64_t c0 = (int64_t)(groups_fast ? blockIdx.x : blockIdx.y) * cg;
-    const int nc = (int)(C - c0 < cg ? C - c0 : cg);
-    const int64_t a0 = tile * MC_TERMS;
-    const int64_t pairs = C * T.cap;   // entries of the Pauli-state arrays
-    if (tid < nc) {
-        spj[tid] = pend[c0 + tid];
-        spq[tid] = pend[C + c0 + tid];
-        sj[tid] = jprop[c0 + tid];
-    }
-    if (tid < MC_ST) mc_bar_init(mc_smem(&full[tid]));
-    if (tid == 0) abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+__global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
+    extern __shared__ uint64_t sF[];          // [n][256]
+    __shared__ uint32_t sw[2][64][8];         // words of a set of planes for the tile, double-buffered
+    __shared__ int s_mf;
+    const int n = T.n, tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
+    const int64_t tile = blockIdx.x, a = tile * MC_TERMS + tid;
+    const int slot = (wi & 3) * 2 + (wi >> 2);   // word of this warp within the tile
+    for (int p = 0; p < n; ++p) sF[p * 256 + tid] = T.F[(int64_t)p * T.cap + a];
+    const uint64_t glo = T.glo[a], ghi = T.ghi[a], v = T.v[a], s = T.s[a];
+    const uint32_t om = T.omega[a];
+    const bool dead = ((om >> 3) & 1u) != 0u;
+    const uint64_t out = dead ? 0ull : ~v & T.nmask;
+    if (tid == 0) s_mf = 0;
     __syncthreads();
-    // err[1] is a one-shot test request (lrs_debug_inject_wait_timeout): block (0, 0)
-    // takes it and makes its first stage expect 16 bytes that no copy delivers, so the
-    // stage's bounded wait runs out
-    uint32_t extra = 0;
-    if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && *(volatile int*)&err[1] != 0) {
-        *(volatile int*)&err[1] = 0;
-        extra = 16;
+    atomicMax(&s_mf, __popcll(out));
+    {
+        float2 b = make_float2(0.f, 0.f);
+        if (!dead) {
+            b = z8_scale(T.coef[a], (int)(om & 7u), __popcll(v) + (int)(om >> 8));
+            b = make_float2(0.5f * b.x, 0.5f * b.y);   // the pass multiplies by +-2 (k_mc_pass)
+        }
+        V.base[(int64_t)((wi >> 2) * 32 + lane) * V.cols + tile * 4 + (wi & 3)] = b;
     }
-    auto issue = [&](int ci, int si) {   // thread 0: chain ci into stage si
-        McStage& S = stage[si];
-        const uint32_t bar = mc_smem(&full[si]);
-        const int pj = spj[ci], j = sj[ci];
-        const int64_t c = c0 + ci;
-        const uint32_t qb = CQ ? MC_TERMS * 12 : MC_TERMS * 16;
-        mc_bar_expect(bar, (uint32_t)(qb + 2 * sizeof(S.fj) + (pj >= 0 ? 2 * sizeof(S.fp) : 0)) + (ci == 0 ? extra : 0u));
-        if (CQ) {
-            mc_bulk_load(mc_smem(S.q), reinterpret_cast<const uint64_t*>(Q) + c * T.cap + a0, MC_TERMS * 8, bar);
-            mc_bulk_load(mc_smem(S.q + MC_TERMS * 8),
-                         reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint64_t*>(Q) + pairs) + c * T.cap + a0,
-                         MC_TERMS * 4, bar);
-        } else {
-            mc_bulk_load(mc_smem(S.q), reinterpret_cast<const ulonglong2*>(Q) + c * T.cap + a0, MC_TERMS * 16, bar);
-        }
-        mc_bulk_load(mc_smem(S.fj), T.F + (int64_t)j * T.cap + a0, sizeof(S.fj), bar);
-        mc_bulk_load(mc_smem(S.mj), T.M + (int64_t)j * T.cap + a0, sizeof(S.mj), bar);
-        if (pj >= 0) {
-            mc_bulk_load(mc_smem(S.fp), T.F + (int64_t)pj * T.cap + a0, sizeof(S.fp), bar);
-            mc_bulk_load(mc_smem(S.mp), T.M + (int64_t)pj * T.cap + a0, sizeof(S.mp), bar);
-        }
+    const int64_t row = V.cols * 2;   // words per plane
+    auto flush = [&](uint32_t* dst, int64_t first, int64_t step, int count, int buf) {
+        for (int e = tid; e < count * 8; e += 256)
+            dst[(first + (int64_t)(e >> 3) * step) * row + tile * 8 + (e & 7)] = sw[buf][e >> 3][e & 7];
     };
-    if (tid == 0)
-        for (int ci = 0; ci < nc && ci < nst; ++ci) issue(ci, ci);
-
-    int tl[MC_TPT];
-    uint64_t glo[MC_TPT], ghi[MC_TPT], s[MC_TPT], nv[MC_TPT], sv[MC_TPT];
-    float2 base[MC_TPT];
-    bool live[MC_TPT];
-#pragma unroll
-    for (int k = 0; k < MC_TPT; ++k) {
-        tl[k] = tid + k * MC_TPB;
-        const int64_t a = a0 + tl[k];
-        glo[k] = T.glo[a];
-        ghi[k] = T.ghi[a];
-        const uint64_t v = T.v[a];
-        s[k] = T.s[a];
-        nv[k] = ~v & T.nmask;
-        sv[k] = s[k] & v;
-        const uint32_t om = T.omega[a];
-        live[k] = ((om >> 3) & 1u) == 0u;
-        base[k] = z8_scale(T.coef[a], (int)(om & 7u), __popcll(v) + (int)(om >> 8));
-    }
-    int ci = 0, si = 0;       // chain, its stage
-    uint32_t ph = 0;          // parity of the stage's current phase
-    for (; ci < nc; ++ci) {
-        const McStage& S = stage[si];
-        if (!mc_bar_wait(mc_smem(&full[si]), ph)) abort_flag = 1;
+    int buf = 0;
+    for (int p = 0; p < n; ++p, buf ^= 1) {
+        const uint64_t Mp = T.M[(int64_t)p * T.cap + a], Fp = sF[p * 256 + tid];
+        for (int q = 0; q < p; ++q) {
+            const uint32_t w = __ballot_sync(0xffffffffu, par64(Mp & sF[q * 256 + tid]));
+            if (lane == 0) sw[buf][q][slot] = w;
+        }
+        const uint32_t lo = __ballot_sync(0xffffffffu, (uint32_t)getb(glo, p));
+        const uint32_t hi =
+            __ballot_sync(0xffffffffu, (uint32_t)getb(ghi, p) ^ par64(Fp & Mp) ^ par64(Fp & s & v));
+        if (lane == 0) {
+            sw[buf][62][slot] = lo;
+            sw[buf][63][slot] = hi;
+        }
         __syncthreads();
-        if (abort_flag) break;   // uniform: read after the barrier
-        const int64_t c = c0 + ci;
-        const int pj = spj[ci], pq = spq[ci], j = sj[ci];
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < MC_TPT; ++k) {
-            uint64_t u, w;
-            uint32_t mu;
-            if (CQ)
-                q_unpack<true>(reinterpret_cast<const uint64_t*>(S.q)[tl[k]],
-                               reinterpret_cast<const uint32_t*>(S.q + MC_TERMS * 8)[tl[k]], u, w, mu);
-            else
-                q_unpack<false>(reinterpret_cast<const ulonglong2*>(S.q)[tl[k]].x,
-                                reinterpret_cast<const ulonglong2*>(S.q)[tl[k]].y, u, w, mu);
-            if (pj >= 0) {   // commit the flip accepted at the previous step
-                const uint64_t Fp = S.fp[tl[k]];
-                mu = (mu + (uint32_t)(getb(glo[k], pj) | (getb(ghi[k], pj) << 1)) + 2u * par64(w & Fp)) & 3u;
-                u ^= Fp;
-                w ^= S.mp[tl[k]];
-            }
-            if (pq >= 0) {   // the second flip of a two-step pass (rows from global memory)
-                const uint64_t Fq = T.F[(int64_t)pq * T.cap + a0 + tl[k]];
-                mu = (mu + (uint32_t)(getb(glo[k], pq) | (getb(ghi[k], pq) << 1)) + 2u * par64(w & Fq)) & 3u;
-                u ^= Fq;
-                w ^= T.M[(int64_t)pq * T.cap + a0 + tl[k]];
-            }
-            if (pj >= 0 || pq >= 0) q_store<CQ>(Q, pairs, c * T.cap + a0 + tl[k], u, w, mu);
-            const uint64_t Fj = S.fj[tl[k]];
-            const uint32_t muy =
-                (mu + (uint32_t)(getb(glo[k], j) | (getb(ghi[k], j) << 1)) + 2u * par64(w & Fj)) & 3u;
-            const uint64_t uy = u ^ Fj, wy = w ^ S.mj[tl[k]];
-            if (live[k] && ((uy ^ s[k]) & nv[k]) == 0) {
-                const uint32_t sign = par64(uy & wy) ^ par64(uy & sv[k]);
-                const float2 t = times_i_pow(base[k], muy + 2u * sign);
-                acc.x += t.x;
-                acc.y += t.y;
-            }
-        }
-        block_sum(acc, red, ci);
-        __syncthreads();   // every thread is done with this stage
-        if (tid == 0 && ci + nst < nc) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            issue(ci + nst, si);
-        }
-        if (++si == nst) {
-            si = 0;
-            ph ^= 1u;
-        }
+        flush(reinterpret_cast<uint32_t*>(V.J), (int64_t)p * (p - 1) / 2, 1, p, buf);
+        if (tid < 16)
+            reinterpret_cast<uint32_t*>(V.D)[(2 * p + (tid >> 3)) * row + tile * 8 + (tid & 7)] = sw[buf][62 + (tid >> 3)][tid & 7];
     }
-    if (ci < nc) {
-        // gave up: wait (bounded) for the copies still in flight into this block's
-        // stages, report, and leave the partial sums unwritten
-        if (tid == 0) {
-            for (int cj = ci; cj < nc && cj < ci + nst; ++cj) {
-                mc_bar_wait(mc_smem(&full[si]), ph);
-                if (++si == nst) {
-                    si = 0;
-                    ph ^= 1u;
-                }
+    const int mf = s_mf;
+    uint64_t ks = out;
+    for (int i = 0; i < mf; ++i, buf ^= 1) {
+        const int k = ks ? ffs64(ks) : -1;   // constraint i of this term: qubit k, or none
+        ks &= ks - 1;
+        for (int p = 0; p < n; ++p) {
+            const uint32_t w = __ballot_sync(0xffffffffu, k >= 0 ? (uint32_t)getb(sF[p * 256 + tid], k) : 0u);
+            if (lane == 0) sw[buf][p][slot] = w;
+        }
+        const uint32_t tg = __ballot_sync(0xffffffffu, k >= 0 ? (uint32_t)getb(s, k) : 0u);
+        if (lane == 0) sw[buf][63][slot] = tg;
+        __syncthreads();
+        flush(reinterpret_cast<uint32_t*>(V.K), (int64_t)i * n, 1, n, buf);
+        if (tid < 8) reinterpret_cast<uint32_t*>(V.target)[i * row + tile * 8 + tid] = sw[buf][63][tid];
+    }
+    if (tid == 0) V.mf[tile] = (uint8_t)mf;
+    if (tid < 8) reinterpret_cast<uint32_t*>(V.J)[mc_pairs(n) * row + tile * 8 + tid] = 0u;
+}
+
+__device__ __forceinline__ uint2 operator^(uint2 a, uint2 b) { return make_uint2(a.x ^ b.x, a.y ^ b.y); }
+__device__ __forceinline__ uint2 operator&(uint2 a, uint2 b) { return make_uint2(a.x & b.x, a.y & b.y); }
+__device__ __forceinline__ uint2 operator|(uint2 a, uint2 b) { return make_uint2(a.x | b.x, a.y | b.y); }
+
+// (lo, hi) += +-(dl, dh) + 2 par, in Z4 planes
+__device__ __forceinline__ void z4_step(uint2& lo, uint2& hi, uint2 dl, uint2 dh, bool minus, uint2 par) {
+    if (minus) dh = dh ^ dl;
+    hi = hi ^ dh ^ (lo & dl) ^ par;
+    lo = lo ^ dl;
+}
+
+// row of J_pq (the zero row for p == q)
+__device__ __forceinline__ int mc_row(int p, int q, int zero) {
+    const int hi = p > q ? p : q, lo = p > q ? q : p;
+    return p == q ? zero : hi * (hi - 1) / 2 + lo;
+}
+
+// State of every (chain, term) at the chains' strings: q(x) by adding the set bits in order,
+// and the syndromes.
+__global__ void __launch_bounds__(MC_TPB) k_mc_start(McView V, int64_t C, uint2* __restrict__ S,
+                                                     const uint64_t* __restrict__ xs, uint64_t nmask, int tbx,
+                                                     int64_t tblocks) {
+    const int tid = threadIdx.x;
+    const int64_t tb = blockIdx.x % tblocks, c = blockIdx.x / tblocks * (MC_TPB / tbx) + tid / tbx;
+    const int64_t col = tb * tbx + tid % tbx;
+    if (c >= C || col >= V.cols) return;
+    const uint64_t x = xs[c] & nmask;
+    const uint2* J = V.J + col;
+    uint2 lo = make_uint2(0u, 0u), hi = lo;
+    for (uint64_t r = x; r; r &= r - 1) {
+        const int p = ffs64(r);
+        uint2 par = make_uint2(0u, 0u);
+        const uint2* Jp = J + (int64_t)(p * (p - 1) / 2) * V.cols;
+        uint64_t below = x & (bit64(p) - 1);
+        while (below) {
+            uint2 t[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                t[u] = make_uint2(0u, 0u);
+                if (below) t[u] = __ldg(Jp + (int64_t)ffs64(below) * V.cols);
+                below &= below - 1;
             }
+            par = par ^ (t[0] ^ t[1]) ^ (t[2] ^ t[3]);
+        }
+        z4_step(lo, hi, __ldg(V.D + (int64_t)(2 * p) * V.cols + col), __ldg(V.D + (int64_t)(2 * p + 1) * V.cols + col), false,
+                par);
+    }
+    const int64_t plane = C * V.cols;
+    uint2* st = S + c * V.cols + col;
+    st[0] = lo;
+    st[plane] = hi;
+    const int mf = V.mf[col >> 2];
+    for (int i = 0; i < mf; ++i) {
+        uint2 y = __ldg(V.target + (int64_t)i * V.cols + col);
+        const uint2* Ki = V.K + (int64_t)i * V.n * V.cols + col;
+        uint64_t r = x;
+        while (r) {
+            uint2 t[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                t[u] = make_uint2(0u, 0u);
+                if (r) t[u] = __ldg(Ki + (int64_t)ffs64(r) * V.cols);
+                r &= r - 1;
+            }
+            y = y ^ (t[0] ^ t[1]) ^ (t[2] ^ t[3]);
+        }
+        st[(MC_PLANES + i) * plane] = y;
+    }
+}
+
+// One pass over the states for one or two steps.  Two steps: the proposals j1 = j_t and
+// j2 = j_{t+1} come from the counter RNG and do not depend on the chain, so one pass forms
+// <y|psi> for every string step t + 1 may propose: y1 = x ^ e_j1, y1 ^ e_j2 (step t accepted)
+// and x ^ e_j2 (rejected); the accept kernel then takes both decisions in order, and the
+// planes of J are read from DRAM once per two steps.  The flips accepted after the previous
+// pass (pend) are applied first, with the parities that pass left.  Each term's
+// contribution and the order of the sums are those of a single step.
+//
+// The FP32 sums are what bounds it: per (term, sum) a sign and live factor (+-2 or +-0, built
+// from two adjacent bits of a nibble and multiplied onto half the coefficient, which is
+// exact), a swap of the two parts, and one fused multiply-add each.
+// At n = 50, chi = 2^20, 256 chains, per step: see the launch below.
+// The block's coefficients (64 rows of tbx columns) are copied once by cp.async.bulk; the wait
+// is bounded (1 s) and a block that gives up sets *err and leaves its sums unwritten.
+template <int STEPS>
+__global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint2* __restrict__ S,
+                                                       const uint64_t* __restrict__ cx,
+                                                       const int32_t* __restrict__ pend,
+                                                       const int32_t* __restrict__ jprop, float2* __restrict__ partial,
+                                                       int cg, int64_t groups, int tbx, int* err) {
+    constexpr int NE = STEPS == 2 ? 3 : 1;   // strings evaluated
+    extern __shared__ __align__(128) float2 sbase[];   // [64][tbx]
+    __shared__ __align__(8) uint64_t full;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t c0 = blockIdx.x % groups * cg, tb = blockIdx.x / groups;
+    const int nc = (int)(C - c0 < cg ? C - c0 : cg);
+    const int nsub = MC_TPB / tbx, tc = tid % tbx;
+    const int64_t col0 = tb * tbx;
+    const int nb = (int)(V.cols - col0 < tbx ? V.cols - col0 : tbx);   // a multiple of 4
+    const uint32_t bar = mc_smem(&full);
+    if (tid == 0) {
+        mc_bar_init(bar);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // err[1] is a one-shot test request (lrs_debug_inject_wait_timeout): block 0 takes it
+        // and expects 16 bytes that no copy delivers, so the bounded wait runs out
+        uint32_t extra = 0;
+        if (blockIdx.x == 0 && *(volatile int*)&err[1] != 0) {
+            *(volatile int*)&err[1] = 0;
+            extra = 16;
+        }
+        mc_bar_expect(bar, (uint32_t)(64 * nb * sizeof(float2)) + extra);
+        for (int r = 0; r < 64; ++r)
+            mc_bulk_load(mc_smem(sbase + r * tbx), V.base + (int64_t)r * V.cols + col0, (uint32_t)(nb * sizeof(float2)), bar);
+    }
+    __syncthreads();
+    if (__syncthreads_or(!mc_bar_wait(bar, 0u))) {
+        // every copy has landed or is waited for once more (bounded) before the block leaves
+        if (tid == 0) {
+            mc_bar_wait(bar, 0u);
             atomicExch(err, 1);
         }
         return;
     }
-    if (tid < nc) {
-        float2 acc = red[tid][0];
-        for (int w2 = 1; w2 < MC_TPB / 32; ++w2) { acc.x += red[tid][w2].x; acc.y += red[tid][w2].y; }
-        partial[(c0 + tid) * n_tiles + tile] = acc;
-    }
-}
-
-// Two steps per pass over the Pauli states.  The proposals j1 = j_t and j2 = j_{t+1}
-// are drawn from the counter RNG and do not depend on the chain, so one pass can form
-// <y|psi> for every string step t + 1 may propose: y1 = x ^ e_j1 (step t), y1 ^ e_j2
-// (step t + 1 after an accepted move) and x ^ e_j2 (after a rejected one), with
-// Q_y1 = Q_x P_j1, Q_y1 P_j2 and Q_x P_j2.  The accept kernel then takes both
-// decisions in order.  Each term's contribution to each sum is the one a single step
-// would add for the same string, in the same order, so the chains are bit-identical to
-// single steps; the pass reads Q once per two steps instead of once per step.
-// Pending flips: both accepted flips of the previous pass, committed in order.
-struct McStage2 {
-    __align__(16) unsigned char q[MC_TERMS * 16];
-    uint64_t f1[MC_TERMS], m1[MC_TERMS], f2[MC_TERMS], m2[MC_TERMS];   // rows F, M of j1, j2
-    uint64_t fp[MC_TERMS], mp[MC_TERMS], fq[MC_TERMS], mq[MC_TERMS];   // rows of the pending flips
-};
-
-// b i^m <0|X(u) Z(w) U_H|s> contribution of one term to a sum over terms (Eq. (amplitude1)).
-__device__ __forceinline__ void mc_add(float2& acc, float2 base, uint64_t s, uint64_t nv, uint64_t sv,
-                                       uint32_t mu, uint64_t u, uint64_t w) {
-    if (((u ^ s) & nv) == 0) {
-        const uint32_t sign = par64(u & w) ^ par64(u & sv);
-        const float2 t = times_i_pow(base, mu + 2u * sign);
-        acc.x += t.x;
-        acc.y += t.y;
-    }
-}
-
-template <bool CQ>
-__global__ void __launch_bounds__(MC_TPB) k_metro_propose2(TermsView T, int64_t C, void* __restrict__ Q,
-                                                           const int32_t* __restrict__ pend,
-                                                           const int32_t* __restrict__ jprop,
-                                                           float2* __restrict__ partial, int64_t n_tiles,
-                                                           int cg, int nst, int* err, int groups_fast) {
-    extern __shared__ __align__(128) unsigned char mc_dyn[];
-    McStage2* stage = reinterpret_cast<McStage2*>(mc_dyn);
-    __shared__ float2 red[3 * MC_CG][MC_TPB / 32];
-    __shared__ int32_t sp1[MC_CG], sp2[MC_CG], sj1[MC_CG], sj2[MC_CG];
-    __shared__ __align__(8) uint64_t full[MC_ST];
-    __shared__ int abort_flag;
-    const int tid = threadIdx.x;
-    const int64_t tile = groups_fast ? blockIdx.y : blockIdx.x;
-    const int64_t c0 = (int64_t)(groups_fast ? blockIdx.x : blockIdx.y) * cg;
-    const int nc = (int)(C - c0 < cg ? C - c0 : cg);
-    const int64_t a0 = tile * MC_TERMS;
-    const int64_t pairs = C * T.cap;
-    if (tid < nc) {
-        sp1[tid] = pend[c0 + tid];
-        sp2[tid] = pend[C + c0 + tid];
-        sj1[tid] = jprop[c0 + tid];
-        sj2[tid] = jprop[C + c0 + tid];
-    }
-    if (tid < MC_ST) mc_bar_init(mc_smem(&full[tid]));
-    if (tid == 0) abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    __syncthreads();
-    // one-shot test request, as in k_metro_propose
-    uint32_t extra = 0;
-    if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0 && *(volatile int*)&err[1] != 0) {
-        *(volatile int*)&err[1] = 0;
-        extra = 16;
-    }
-    auto issue = [&](int ci, int si) {   // thread 0: chain ci into stage si
-        McStage2& S = stage[si];
-        const uint32_t bar = mc_smem(&full[si]);
-        const int p1 = sp1[ci], p2 = sp2[ci], j1 = sj1[ci], j2 = sj2[ci];
-        const int64_t c = c0 + ci;
-        const uint32_t qb = CQ ? MC_TERMS * 12 : MC_TERMS * 16;
-        const uint32_t rb = (uint32_t)sizeof(S.f1);
-        mc_bar_expect(bar, qb + 4 * rb + (p1 >= 0 ? 2 * rb : 0u) + (p2 >= 0 ? 2 * rb : 0u) + (ci == 0 ? extra : 0u));
-        if (CQ) {
-            mc_bulk_load(mc_smem(S.q), reinterpret_cast<const uint64_t*>(Q) + c * T.cap + a0, MC_TERMS * 8, bar);
-            mc_bulk_load(mc_smem(S.q + MC_TERMS * 8),
-                         reinterpret_cast<const uint32_t*>(reinterpret_cast<const uint64_t*>(Q) + pairs) + c * T.cap + a0,
-                         MC_TERMS * 4, bar);
-        } else {
-            mc_bulk_load(mc_smem(S.q), reinterpret_cast<const ulonglong2*>(Q) + c * T.cap + a0, MC_TERMS * 16, bar);
-        }
-        mc_bulk_load(mc_smem(S.f1), T.F + (int64_t)j1 * T.cap + a0, rb, bar);
-        mc_bulk_load(mc_smem(S.m1), T.M + (int64_t)j1 * T.cap + a0, rb, bar);
-        mc_bulk_load(mc_smem(S.f2), T.F + (int64_t)j2 * T.cap + a0, rb, bar);
-        mc_bulk_load(mc_smem(S.m2), T.M + (int64_t)j2 * T.cap + a0, rb, bar);
-        if (p1 >= 0) {
-            mc_bulk_load(mc_smem(S.fp), T.F + (int64_t)p1 * T.cap + a0, rb, bar);
-            mc_bulk_load(mc_smem(S.mp), T.M + (int64_t)p1 * T.cap + a0, rb, bar);
-        }
-        if (p2 >= 0) {
-            mc_bulk_load(mc_smem(S.fq), T.F + (int64_t)p2 * T.cap + a0, rb, bar);
-            mc_bulk_load(mc_smem(S.mq), T.M + (int64_t)p2 * T.cap + a0, rb, bar);
-        }
-    };
-    if (tid == 0)
-        for (int ci = 0; ci < nc && ci < nst; ++ci) issue(ci, ci);
-
-    int tl[MC_TPT];
-    uint64_t glo[MC_TPT], ghi[MC_TPT], s[MC_TPT], nv[MC_TPT], sv[MC_TPT];
-    float2 base[MC_TPT];
-    bool live[MC_TPT];
-#pragma unroll
-    for (int k = 0; k < MC_TPT; ++k) {
-        tl[k] = tid + k * MC_TPB;
-        const int64_t a = a0 + tl[k];
-        glo[k] = T.glo[a];
-        ghi[k] = T.ghi[a];
-        const uint64_t v = T.v[a];
-        s[k] = T.s[a];
-        nv[k] = ~v & T.nmask;
-        sv[k] = s[k] & v;
-        const uint32_t om = T.omega[a];
-        live[k] = ((om >> 3) & 1u) == 0u;
-        base[k] = z8_scale(T.coef[a], (int)(om & 7u), __popcll(v) + (int)(om >> 8));
-    }
-    int ci = 0, si = 0;
-    uint32_t ph = 0;
-    for (; ci < nc; ++ci) {
-        const McStage2& S = stage[si];
-        if (!mc_bar_wait(mc_smem(&full[si]), ph)) abort_flag = 1;
-        __syncthreads();
-        if (abort_flag) break;   // uniform: read after the barrier
-        const int64_t c = c0 + ci;
-        const int p1 = sp1[ci], p2 = sp2[ci], j1 = sj1[ci], j2 = sj2[ci];
-        float2 acc1 = make_float2(0.f, 0.f), acc2a = acc1, acc2r = acc1;
-#pragma unroll
-        for (int k = 0; k < MC_TPT; ++k) {
-            uint64_t u, w;
-            uint32_t mu;
-            if (CQ)
-                q_unpack<true>(reinterpret_cast<const uint64_t*>(S.q)[tl[k]],
-                               reinterpret_cast<const uint32_t*>(S.q + MC_TERMS * 8)[tl[k]], u, w, mu);
-            else
-                q_unpack<false>(reinterpret_cast<const ulonglong2*>(S.q)[tl[k]].x,
-                                reinterpret_cast<const ulonglong2*>(S.q)[tl[k]].y, u, w, mu);
-            if (p1 >= 0) {   // commit the flips accepted in the previous pass, in order
-                const uint64_t Fp = S.fp[tl[k]];
-                mu = (mu + (uint32_t)(getb(glo[k], p1) | (getb(ghi[k], p1) << 1)) + 2u * par64(w & Fp)) & 3u;
-                u ^= Fp;
-                w ^= S.mp[tl[k]];
+    const bool in = tc < nb;
+    const int64_t col = col0 + (in ? tc : 0), plane = C * V.cols, n_tiles = V.cols >> 2;
+    const int mf = V.mf[col >> 2];
+    const int mfw = __reduce_max_sync(0xffffffffu, mf);
+    const int zero = mc_pairs(V.n);
+    const uint2* J = V.J + col;
+    const uint2* D = V.D + col;
+    const float2* bp = sbase + tc;
+    const uint2 none = make_uint2(0u, 0u);
+    for (int i0 = 0; i0 < nc; i0 += nsub) {
+        const int ci = i0 + tid / tbx;
+        const bool on = in && ci < nc;
+        const int64_t c = c0 + (ci < nc ? ci : 0);
+        const uint64_t x = cx[c];
+        const int p1 = pend[c], p2 = pend[C + c], j1 = jprop[c], j2 = STEPS == 2 ? jprop[C + c] : 0;
+        uint2* st = S + c * V.cols + col;
+        uint2 lo = st[0], hi = st[plane];
+        const bool moved = p1 >= 0 || p2 >= 0;
+        if (moved) {   // the flips accepted after the previous pass, in order
+            uint64_t xo = x ^ (p1 >= 0 ? bit64(p1) : 0ull) ^ (p2 >= 0 ? bit64(p2) : 0ull);
+            uint2 par2 = p2 >= 0 ? st[3 * plane] : none;
+            if (p1 >= 0) {
+                z4_step(lo, hi, __ldg(D + (int64_t)(2 * p1) * V.cols), __ldg(D + (int64_t)(2 * p1 + 1) * V.cols), getb(xo, p1) != 0,
+                        st[2 * plane]);
+                xo ^= bit64(p1);
+                if (p2 >= 0) par2 = par2 ^ __ldg(J + (int64_t)mc_row(p1, p2, zero) * V.cols);
             }
-            if (p2 >= 0) {
-                const uint64_t Fq = S.fq[tl[k]];
-                mu = (mu + (uint32_t)(getb(glo[k], p2) | (getb(ghi[k], p2) << 1)) + 2u * par64(w & Fq)) & 3u;
-                u ^= Fq;
-                w ^= S.mq[tl[k]];
+            if (p2 >= 0)
+                z4_step(lo, hi, __ldg(D + (int64_t)(2 * p2) * V.cols), __ldg(D + (int64_t)(2 * p2 + 1) * V.cols), getb(xo, p2) != 0,
+                        par2);
+            if (on) {
+                st[0] = lo;
+                st[plane] = hi;
             }
-            if (p1 >= 0 || p2 >= 0) q_store<CQ>(Q, pairs, c * T.cap + a0 + tl[k], u, w, mu);
-            if (!live[k]) continue;
-            const uint64_t F1 = S.f1[tl[k]], M1 = S.m1[tl[k]], F2 = S.f2[tl[k]], M2 = S.m2[tl[k]];
-            const uint32_t g1 = (uint32_t)(getb(glo[k], j1) | (getb(ghi[k], j1) << 1));
-            const uint32_t g2 = (uint32_t)(getb(glo[k], j2) | (getb(ghi[k], j2) << 1));
-            // y1 = x ^ e_j1
-            const uint32_t mu1 = (mu + g1 + 2u * par64(w & F1)) & 3u;
-            const uint64_t u1 = u ^ F1, w1 = w ^ M1;
-            mc_add(acc1, base[k], s[k], nv[k], sv[k], mu1, u1, w1);
-            // y1 ^ e_j2 (step t accepted)
-            mc_add(acc2a, base[k], s[k], nv[k], sv[k], (mu1 + g2 + 2u * par64(w1 & F2)) & 3u, u1 ^ F2, w1 ^ M2);
-            // x ^ e_j2 (step t rejected)
-            mc_add(acc2r, base[k], s[k], nv[k], sv[k], (mu + g2 + 2u * par64(w & F2)) & 3u, u ^ F2, w ^ M2);
         }
-        block_sum(acc1, red, 3 * ci);
-        block_sum(acc2a, red, 3 * ci + 1);
-        block_sum(acc2r, red, 3 * ci + 2);
-        __syncthreads();   // every thread is done with this stage
-        if (tid == 0 && ci + nst < nc) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            issue(ci + nst, si);
+        // J_j . x for the proposals (the zero row stands in for q = j and past the last bit)
+        uint2 par1 = none, par2 = none;
+        for (uint64_t r = x; r;) {
+            uint2 t1[4], t2[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q = r ? ffs64(r) : j1;
+                t1[u] = __ldg(J + (int64_t)mc_row(j1, q, zero) * V.cols);
+                if (STEPS == 2) t2[u] = __ldg(J + (int64_t)(r ? mc_row(j2, q, zero) : zero) * V.cols);
+                r &= r - 1;
+            }
+            par1 = par1 ^ (t1[0] ^ t1[1]) ^ (t1[2] ^ t1[3]);
+            if (STEPS == 2) par2 = par2 ^ (t2[0] ^ t2[1]) ^ (t2[2] ^ t2[3]);
         }
-        if (++si == nst) {
-            si = 0;
-            ph ^= 1u;
+        if (on) {
+            st[2 * plane] = par1;
+            if (STEPS == 2) st[3 * plane] = par2;
         }
-    }
-    if (ci < nc) {
-        // gave up: wait (bounded) for the copies still in flight, report, and leave the
-        // partial sums unwritten
-        if (tid == 0) {
-            for (int cj = ci; cj < nc && cj < ci + nst; ++cj) {
-                mc_bar_wait(mc_smem(&full[si]), ph);
-                if (++si == nst) {
-                    si = 0;
-                    ph ^= 1u;
+        // phases of y1, y1 ^ e_j2, x ^ e_j2
+        uint2 L[NE], H[NE], dead[NE];
+        {
+            const uint2 dl = __ldg(D + (int64_t)(2 * j1) * V.cols), dh = __ldg(D + (int64_t)(2 * j1 + 1) * V.cols);
+            L[0] = lo;
+            H[0] = hi;
+            z4_step(L[0], H[0], dl, dh, getb(x, j1) != 0, par1);
+            dead[0] = none;
+        }
+        if (STEPS == 2) {
+            const uint2 dl = __ldg(D + (int64_t)(2 * j2) * V.cols), dh = __ldg(D + (int64_t)(2 * j2 + 1) * V.cols);
+            const uint2 j12 = __ldg(J + (int64_t)mc_row(j1, j2, zero) * V.cols);
+            L[1] = L[0];
+            H[1] = H[0];
+            z4_step(L[1], H[1], dl, dh, getb(x ^ bit64(j1), j2) != 0, par2 ^ j12);
+            L[NE - 1] = lo;
+            H[NE - 1] = hi;
+            z4_step(L[NE - 1], H[NE - 1], dl, dh, getb(x, j2) != 0, par2);
+            dead[1] = none;
+            dead[NE - 1] = none;
+        }
+#pragma unroll 2
+        for (int i = 0; i < mfw; ++i) {
+            if (i >= mf) continue;   // this tile has fewer
+            const uint2* Ki = V.K + (int64_t)i * V.n * V.cols + col;
+            uint2 y = st[(MC_PLANES + i) * plane];
+            const uint2 k1 = __ldg(Ki + (int64_t)j1 * V.cols), k2 = STEPS == 2 ? __ldg(Ki + (int64_t)j2 * V.cols) : none;
+            if (moved) {
+                if (p1 >= 0) y = y ^ __ldg(Ki + (int64_t)p1 * V.cols);
+                if (p2 >= 0) y = y ^ __ldg(Ki + (int64_t)p2 * V.cols);
+                if (on) st[(MC_PLANES + i) * plane] = y;
+            }
+            dead[0] = dead[0] | (y ^ k1);
+            if (STEPS == 2) {
+                dead[1] = dead[1] | (y ^ k1 ^ k2);
+                dead[NE - 1] = dead[NE - 1] | (y ^ k2);
+            }
+        }
+        // sums
+        bool some = false;
+#pragma unroll
+        for (int e = 0; e < NE; ++e) some = some || (dead[e].x & dead[e].y) != 0xffffffffu;
+        float2 f[NE], u[NE];
+#pragma unroll
+        for (int e = 0; e < NE; ++e) f[e] = u[e] = make_float2(0.f, 0.f);
+        if (__any_sync(0xffffffffu, some)) {
+#pragma unroll 1
+            for (int it = 0; it < 4; ++it) {
+                // leaves l = l0 + 4 t, l0 = bits 0 and 1 of l
+                const int l0 = (it >> 1) + 2 * (it & 1);
+                uint32_t N0[NE], N1[NE];   // nibble t: live, phase bit 1, phase bit 0
+#pragma unroll
+                for (int e = 0; e < NE; ++e) {
+                    constexpr uint32_t one = 0x11111111u;
+                    N0[e] = (~dead[e].x >> l0 & one) | (H[e].x >> l0 & one) << 1 | (L[e].x >> l0 & one) << 2;
+                    N1[e] = (~dead[e].y >> l0 & one) | (H[e].y >> l0 & one) << 1 | (L[e].y >> l0 & one) << 2;
+                }
+                const float2* b0 = bp + l0 * tbx;
+                float2 v[NE][8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    const float2 ba = b0[4 * t * tbx], bb = b0[(32 + 4 * t) * tbx];
+#pragma unroll
+                    for (int e = 0; e < NE; ++e) {
+                        // b i^m, m = 2 hi + lo: (x, y) or (-y, x), times (-1)^hi
+                        const float fa = __uint_as_float((N0[e] << (30 - 4 * t)) & 0xC0000000u);
+                        const float fb = __uint_as_float((N1[e] << (30 - 4 * t)) & 0xC0000000u);
+                        const bool sa = (N0[e] & (4u << (4 * t))) != 0, sb = (N1[e] & (4u << (4 * t))) != 0;
+                        const float rx = fa * (sa ? -ba.y : ba.x), ry = fa * (sa ? ba.x : ba.y);
+                        v[e][t].x = fmaf(fb, sb ? -bb.y : bb.x, rx);
+                        v[e][t].y = fmaf(fb, sb ? bb.x : bb.y, ry);
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < NE; ++e) {
+#pragma unroll
+                    for (int h = 4; h > 0; h >>= 1)   // bits 4, 3, 2 of l
+#pragma unroll
+                        for (int t = 0; t < h; ++t) {
+                            v[e][t].x += v[e][t + h].x;
+                            v[e][t].y += v[e][t + h].y;
+                        }
+                    // bit 1, then bit 0
+                    if (it & 1) {
+                        u[e].x += v[e][0].x;
+                        u[e].y += v[e][0].y;
+                    } else {
+                        u[e] = v[e][0];
+                    }
+                    if (it == 1) f[e] = u[e];
+                    if (it == 3) {
+                        f[e].x += u[e].x;
+                        f[e].y += u[e].y;
+                    }
                 }
             }
-            atomicExch(err, 1);
         }
-        return;
-    }
-    for (int e = tid; e < 3 * nc; e += MC_TPB) {   // sum r of chain cc: [r][chain][tile]
-        const int cc = e / 3, r = e - 3 * cc;
-        float2 acc = red[e][0];
-        for (int w2 = 1; w2 < MC_TPB / 32; ++w2) { acc.x += red[e][w2].x; acc.y += red[e][w2].y; }
-        partial[((int64_t)r * C + c0 + cc) * n_tiles + tile] = acc;
+        // the four columns of the tile in order
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            float2 acc = f[e];
+#pragma unroll
+            for (int w = 1; w < 4; ++w) {
+                acc.x += __shfl_down_sync(0xffffffffu, f[e].x, w);
+                acc.y += __shfl_down_sync(0xffffffffu, f[e].y, w);
+            }
+            if (on && (lane & 3) == 0) partial[((int64_t)e * C + c) * n_tiles + (col >> 2)] = acc;
+        }
     }
 }
 
@@ -603,7 +593,9 @@ __global__ void k_mh_accept(const double* __restrict__ ampy, const uint64_t* __r
 
 // Term-sharded steps: the FP64 sum over tiles of each chain's partial <y|psi_shard>
 // (not squared: the shards' sums add before P(y) is formed).
-__global__ void k_metro_partial_out(const float2* __restrict__ partial, int64_t n_tiles, double* __restrict__ amp) {
+// The pass has applied the pending flips, so they are cleared.
+__global__ void k_metro_partial_out(const float2* __restrict__ partial, int64_t n_tiles, double* __restrict__ amp,
+                                    int32_t* pend, int64_t C) {
     const int64_t c = blockIdx.x;
     double re = 0.0, im = 0.0;
     for (int64_t t = threadIdx.x; t < n_tiles; t += blockDim.x) {
@@ -625,6 +617,8 @@ __global__ void k_metro_partial_out(const float2* __restrict__ partial, int64_t 
     if (threadIdx.x == 0) {
         amp[2 * c] = sre[0];
         amp[2 * c + 1] = sim[0];
+        pend[c] = -1;
+        pend[C + c] = -1;
     }
 }
 
@@ -671,15 +665,107 @@ __global__ void k_metro_out(int64_t C, const uint64_t* cx, const double* cp, uin
 
 }  // namespace
 
-lrs_status launch_chains_init(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) {
-    // Q of every (chain, term) and <x_c|psi> by the amplitude kernel (Four-Russians
-    // tables of the Pauli accumulator), then the chain scalars
+// Pointers into ctx->mc_planes (layout of McView).
+static size_t mc_layout(const lrs_ctx* ctx, McView* V) {
+    const int n = ctx->n;
+    const int64_t cols = ctx->cap / 64;
+    const size_t plane = (size_t)cols * sizeof(uint2);
+    char* p = (char*)ctx->mc_planes;
+    size_t at = 0;
+    auto take = [&](size_t planes) {
+        char* q = p + at;
+        at += planes * plane;
+        return q;
+    };
+    McView v;
+    v.n = n;
+    v.cols = cols;
+    v.base = (float2*)take(64);
+    v.J = (uint2*)take(mc_pairs(n) + 1);
+    v.D = (uint2*)take(2 * n);
+    v.K = (uint2*)take((size_t)n * n);
+    v.target = (uint2*)take(n);
+    v.mf = (uint8_t*)take(1);   // cols / 4 bytes
+    if (V) *V = v;
+    return at;
+}
+
+size_t mc_planes_bytes(const lrs_ctx* ctx) { return mc_layout(ctx, nullptr); }
+size_t mc_state_bytes(const lrs_ctx* ctx, int64_t chains) {
+    return (size_t)(MC_PLANES + ctx->n) * chains * (ctx->cap / 64) * sizeof(uint2);
+}
+
+// Columns per block: 128, fewer (a power of two) for a context of fewer terms, whose
+// blocks then take several chains at a time.
+static int mc_columns(int64_t cols) {
+    int t = MC_TPB;
+    while (t > 4 && t / 2 >= cols) t /= 2;
+    return t;
+}
+
+// States and P(x) of the chains at strings x.
+static lrs_status mc_start(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) {
+    McView V;
+    mc_layout(ctx, &V);
     const int64_t C = ctx->n_chains;
+    const int tbx = mc_columns(V.cols), nsub = MC_TPB / tbx;
+    const int64_t tblocks = (V.cols + tbx - 1) / tbx, blocks = tblocks * ((C + nsub - 1) / nsub);
+    if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "chain start grid too large");
+    k_mc_start<<<(unsigned)blocks, MC_TPB, 0, st>>>(V, C, (uint2*)ctx->Q, x, ctx->nmask, tbx, tblocks);
+    LRS_LAUNCH_CHECK("chain start kernel");
     double* amp = nullptr;
-    lrs_status rc = launch_amplitude_q(ctx, x, C, ctx->Q, &amp, st);
+    lrs_status rc = launch_amplitude_start(ctx, x, C, &amp, st);
     if (rc != LRS_OK) return rc;
     k_chains_set<<<(unsigned)((C + 127) / 128), 128, 0, st>>>(amp, C, x, ctx->nmask, ctx->cx, ctx->cp, ctx->pend);
     LRS_LAUNCH_CHECK("chains_set kernel");
+    return LRS_OK;
+}
+
+lrs_status launch_chains_init(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) {
+    // the planes of the current terms, then the chains' states and probabilities
+    McView V;
+    mc_layout(ctx, &V);
+    const size_t smem = (size_t)ctx->n * 256 * sizeof(uint64_t);
+    if (!lrs_capturing(st))
+        LRS_CUDA(cudaFuncSetAttribute(k_mc_planes, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(62 * 256 * sizeof(uint64_t))));
+    k_mc_planes<<<(unsigned)(ctx->cap / MC_TERMS), 256, smem, st>>>(ctx->view(), V);
+    LRS_LAUNCH_CHECK("chain planes kernel");
+    return mc_start(ctx, x, st);
+}
+
+// One pass of `steps` (1 or 2) steps.
+static lrs_status mc_pass(lrs_ctx* ctx, int steps, const int32_t* jprop, float2* partial, cudaStream_t st) {
+    McView V;
+    mc_layout(ctx, &V);
+    const int64_t C = ctx->n_chains;
+    const int tbx = mc_columns(V.cols), nsub = MC_TPB / tbx;
+    const int64_t tblocks = (V.cols + tbx - 1) / tbx;
+    // chains per block: up to the tuned number, fewer while the grid is under four
+    // rounds of three blocks per SM (a block's coefficients are one copy of 64 KB)
+    const int64_t want = ((int64_t)12 * ctx->sm_count + tblocks - 1) / tblocks;
+    int64_t cg = (C + want - 1) / want;
+    if (cg < nsub) cg = nsub;
+    if (cg > ctx->tune_mc_cg) cg = ctx->tune_mc_cg;
+    const int64_t groups = (C + cg - 1) / cg, blocks = tblocks * groups;
+    if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "Metropolis grid too large");
+    const size_t smem = (size_t)64 * tbx * sizeof(float2);
+    if (steps == 2)
+        k_mc_pass<2><<<(unsigned)blocks, MC_TPB, smem, st>>>(V, C, (uint2*)ctx->Q, ctx->cx, ctx->pend, jprop, partial,
+                                                             (int)cg, groups, tbx, ctx->mc_err_d);
+    else
+        k_mc_pass<1><<<(unsigned)blocks, MC_TPB, smem, st>>>(V, C, (uint2*)ctx->Q, ctx->cx, ctx->pend, jprop, partial,
+                                                             (int)cg, groups, tbx, ctx->mc_err_d);
+    LRS_LAUNCH_CHECK("metropolis pass kernel");
+    return LRS_OK;
+}
+
+static lrs_status mc_attributes(cudaStream_t st) {
+    // inside a graph capture the attributes were set by an earlier uncaptured call
+    if (lrs_capturing(st)) return LRS_OK;
+    const int most = (int)(64 * MC_TPB * sizeof(float2));
+    LRS_CUDA(cudaFuncSetAttribute(k_mc_pass<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    LRS_CUDA(cudaFuncSetAttribute(k_mc_pass<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     return LRS_OK;
 }
 
@@ -688,23 +774,11 @@ static lrs_status enqueue_steps(lrs_ctx* ctx, int64_t t0, int64_t count, float2*
                                 uint64_t* trace, cudaStream_t st) {
     const int64_t C = ctx->n_chains;
     const int64_t n_tiles = ctx->cap / MC_TERMS;
-    const int cg = (int)ctx->tune_mc_cg;
-    // chain groups fastest (the rows of a tile are read from DRAM once per step, not once
-    // per group); tiles along x when they exceed the grid's y limit
-    const int64_t groups = (C + cg - 1) / cg;
-    const int gf = n_tiles <= 65535 ? 1 : 0;
-    dim3 grid = gf ? dim3((unsigned)groups, (unsigned)n_tiles) : dim3((unsigned)n_tiles, (unsigned)groups);
-    const int nst = (int)ctx->tune_mc_stages;
+    lrs_status rc;
     int64_t t = t0;
     if (ctx->tune_mc_lookahead == 2) {
         for (; t + 1 < t0 + count; t += 2) {
-            if (q_compact(ctx->n))
-                k_metro_propose2<true><<<grid, MC_TPB, nst * sizeof(McStage2), st>>>(
-                    ctx->view(), C, ctx->Q, ctx->pend, jprop, partial, n_tiles, cg, nst, ctx->mc_err_d, gf);
-            else
-                k_metro_propose2<false><<<grid, MC_TPB, nst * sizeof(McStage2), st>>>(
-                    ctx->view(), C, ctx->Q, ctx->pend, jprop, partial, n_tiles, cg, nst, ctx->mc_err_d, gf);
-            LRS_LAUNCH_CHECK("metropolis two-step propose kernel");
+            if ((rc = mc_pass(ctx, 2, jprop, partial, st)) != LRS_OK) return rc;
             k_metro_accept2<<<(unsigned)C, 256, 0, st>>>(partial, n_tiles, ctx->mc_par, t, ctx->n, ctx->cx,
                                                           ctx->cp, ctx->pend, jprop,
                                                           trace ? trace + t * C : nullptr, C);
@@ -712,13 +786,7 @@ static lrs_status enqueue_steps(lrs_ctx* ctx, int64_t t0, int64_t count, float2*
         }
     }
     for (; t < t0 + count; ++t) {
-        if (q_compact(ctx->n))
-            k_metro_propose<true><<<grid, MC_TPB, nst * sizeof(McStage), st>>>(
-                ctx->view(), C, ctx->Q, ctx->pend, jprop, partial, n_tiles, cg, nst, ctx->mc_err_d, gf);
-        else
-            k_metro_propose<false><<<grid, MC_TPB, nst * sizeof(McStage), st>>>(
-                ctx->view(), C, ctx->Q, ctx->pend, jprop, partial, n_tiles, cg, nst, ctx->mc_err_d, gf);
-        LRS_LAUNCH_CHECK("metropolis propose kernel");
+        if ((rc = mc_pass(ctx, 1, jprop, partial, st)) != LRS_OK) return rc;
         k_metro_accept<<<(unsigned)C, 256, 0, st>>>(partial, n_tiles, ctx->mc_par, t, ctx->n, ctx->cx,
                                                      ctx->cp, ctx->pend, jprop,
                                                      trace ? trace + t * C : nullptr, C);
@@ -730,7 +798,7 @@ static lrs_status enqueue_steps(lrs_ctx* ctx, int64_t t0, int64_t count, float2*
 // One CUDA graph holding LRS_MC_GRAPH_STEPS steps followed by step0 += steps;
 // rebuilt whenever the buffers it was captured with change.
 static lrs_status mc_graph(lrs_ctx* ctx, float2* partial, int32_t* jprop, cudaGraphExec_t* out) {
-    const void* key[6] = {partial, jprop, ctx->Q, ctx->F,
+    const void* key[6] = {partial, jprop, ctx->Q, ctx->mc_planes,
                           (void*)(intptr_t)(((ctx->n_chains * 128 + ctx->tune_mc_cg) * 8 + ctx->tune_mc_stages) * 4 +
                                             ctx->tune_mc_lookahead),
                           (void*)(intptr_t)ctx->cap};
@@ -792,19 +860,9 @@ lrs_status launch_metropolis(lrs_ctx* ctx, int64_t steps, uint64_t seed, int64_t
         *(volatile int*)ctx->mc_err_h = 0;
         return lrs_fail(LRS_ERR_TIMEOUT, "a Metropolis propose kernel gave up waiting for its copies");
     }
-    // inside a graph capture: the attributes were set by an earlier uncaptured call, and
-    // the steps are captured as plain launches (no nested graph)
+    // inside a graph capture the steps are captured as plain launches (no nested graph)
     const bool capturing = lrs_capturing(st);
-    if (!capturing) {
-        LRS_CUDA(cudaFuncSetAttribute(k_metro_propose<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(MC_ST * sizeof(McStage))));
-        LRS_CUDA(cudaFuncSetAttribute(k_metro_propose<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(MC_ST * sizeof(McStage))));
-        LRS_CUDA(cudaFuncSetAttribute(k_metro_propose2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(MC_ST * sizeof(McStage2))));
-        LRS_CUDA(cudaFuncSetAttribute(k_metro_propose2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(MC_ST * sizeof(McStage2))));
-    }
+    if ((rc = mc_attributes(st)) != LRS_OK) return rc;
     float2* partial = (float2*)scr;
     int32_t* jprop = (int32_t*)((char*)scr + ((part_bytes + 255) & ~(size_t)255));
     k_mc_set<<<1, 1, 0, st>>>(ctx->mc_par, seed, step0);
@@ -843,29 +901,13 @@ lrs_status launch_metropolis_propose(lrs_ctx* ctx, uint64_t seed, int64_t step, 
         *(volatile int*)ctx->mc_err_h = 0;
         return lrs_fail(LRS_ERR_TIMEOUT, "a Metropolis propose kernel gave up waiting for its copies");
     }
-    if (!lrs_capturing(st)) {
-        LRS_CUDA(cudaFuncSetAttribute(k_metro_propose<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(MC_ST * sizeof(McStage))));
-        LRS_CUDA(cudaFuncSetAttribute(k_metro_propose<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(MC_ST * sizeof(McStage))));
-    }
+    if ((rc = mc_attributes(st)) != LRS_OK) return rc;
     k_mc_set<<<1, 1, 0, st>>>(ctx->mc_par, seed, step);
     k_metro_first<<<(unsigned)((C + 127) / 128), 128, 0, st>>>(C, ctx->mc_par, ctx->n, ctx->jbuf, nullptr);
     LRS_LAUNCH_CHECK("metropolis first kernel");
-    const int cg = (int)ctx->tune_mc_cg;
-    const int64_t groups = (C + cg - 1) / cg;
-    const int gf = n_tiles <= 65535 ? 1 : 0;
-    dim3 grid = gf ? dim3((unsigned)groups, (unsigned)n_tiles) : dim3((unsigned)n_tiles, (unsigned)groups);
-    const int nst = (int)ctx->tune_mc_stages;
     float2* partial = (float2*)scr;
-    if (q_compact(ctx->n))
-        k_metro_propose<true><<<grid, MC_TPB, nst * sizeof(McStage), st>>>(
-            ctx->view(), C, ctx->Q, ctx->pend, ctx->jbuf, partial, n_tiles, cg, nst, ctx->mc_err_d, gf);
-    else
-        k_metro_propose<false><<<grid, MC_TPB, nst * sizeof(McStage), st>>>(
-            ctx->view(), C, ctx->Q, ctx->pend, ctx->jbuf, partial, n_tiles, cg, nst, ctx->mc_err_d, gf);
-    LRS_LAUNCH_CHECK("metropolis propose kernel");
-    k_metro_partial_out<<<(unsigned)C, 256, 0, st>>>(partial, n_tiles, amp);
+    if ((rc = mc_pass(ctx, 1, ctx->jbuf, partial, st)) != LRS_OK) return rc;
+    k_metro_partial_out<<<(unsigned)C, 256, 0, st>>>(partial, n_tiles, amp, ctx->pend, C);
     LRS_LAUNCH_CHECK("metropolis partial amplitude kernel");
     return LRS_OK;
 }
@@ -920,19 +962,15 @@ lrs_status launch_metropolis_learned(lrs_ctx* ctx, lrs_mlp* mlp, int64_t steps, 
     return LRS_OK;
 }
 
-// Rebuild Q for the chains' current strings (after learned moves).  The strings are
+// Rebuild the states for the chains' current strings (after learned moves).  The strings are
 // copied into the learned proposal's buffer (free at this point) because chains_set
 // rewrites cx.
 lrs_status launch_chains_refresh(lrs_ctx* ctx, cudaStream_t st) {
     const int64_t C = ctx->n_chains;
     if (!ctx->ybuf || ctx->mh_cap < C) return lrs_fail(LRS_ERR_STATE, "chain refresh without a learned-move buffer");
     LRS_CUDA(cudaMemcpyAsync(ctx->ybuf, ctx->cx, (size_t)C * 8, cudaMemcpyDeviceToDevice, st));
-    double* amp = nullptr;
-    lrs_status rc = launch_amplitude_q(ctx, ctx->ybuf, C, ctx->Q, &amp, st);
+    const lrs_status rc = mc_start(ctx, ctx->ybuf, st);
     if (rc != LRS_OK) return rc;
-    k_chains_set<<<(unsigned)((C + 127) / 128), 128, 0, st>>>(amp, C, ctx->ybuf, ctx->nmask, ctx->cx, ctx->cp,
-                                                            ctx->pend);
-    LRS_LAUNCH_CHECK("chains refresh set kernel");
     ctx->q_stale = false;
     return LRS_OK;
 }

@@ -288,6 +288,9 @@ static void free_terms(lrs_ctx* c) {
 }
 
 static void free_chains(lrs_ctx* c) {
+    cudaFree(c->mc_planes);
+    c->mc_planes = nullptr;
+    c->mc_planes_bytes = 0;
     cudaFree(c->Q); cudaFree(c->cx); cudaFree(c->cp); cudaFree(c->pend);
     c->Q = nullptr; c->cx = nullptr; c->cp = nullptr; c->pend = nullptr;
     c->Q_bytes = 0; c->chains_cap = 0; c->n_chains = 0;
@@ -871,8 +874,9 @@ extern "C" lrs_status lrs_chains_init(lrs_ctx* c, int64_t n_chains, const uint64
     if (n_chains < 1 || !x) return lrs_fail(LRS_ERR_ARG, "bad chains");
     if (n_chains > 65535) return lrs_fail(LRS_ERR_ARG, "at most 65535 chains");
     LRS_CUDA(cudaSetDevice(c->device));
-    const size_t qb = (size_t)n_chains * c->cap * q_bytes(c->n);
-    lrs_status rc = lrs_ensure((void**)&c->Q, &c->Q_bytes, qb);
+    lrs_status rc = lrs_ensure((void**)&c->Q, &c->Q_bytes, mc_state_bytes(c, n_chains));
+    if (rc != LRS_OK) return rc;
+    rc = lrs_ensure(&c->mc_planes, &c->mc_planes_bytes, mc_planes_bytes(c));
     if (rc != LRS_OK) return rc;
     if (n_chains > c->chains_cap) {
         cudaFree(c->cx); cudaFree(c->cp); cudaFree(c->pend);

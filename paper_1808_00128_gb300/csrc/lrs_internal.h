@@ -111,13 +111,15 @@ struct lrs_ctx {
 
     // Metropolis chains
     int64_t n_chains = 0;
-    void* Q = nullptr;              // [chain][cap] Pauli states (q_store layout)
+    void* Q = nullptr;              // bit-plane states of every (chain, term) (k_metropolis.cu)
     size_t Q_bytes = 0;
+    void* mc_planes = nullptr;      // bit-planes of the terms, made by lrs_chains_init
+    size_t mc_planes_bytes = 0;
     uint64_t* cx = nullptr;         // [chain] current x
     double* cp = nullptr;           // [chain] P(x) (unnormalised)
     int32_t* pend = nullptr;        // [2][chain] pending accepted flips, committed in order (-1 none)
     int64_t chains_cap = 0;
-    bool q_stale = false;           // x moved by learned proposals: Q must be rebuilt
+    bool q_stale = false;           // x moved by learned proposals: the states must be rebuilt
     McParams* mc_par = nullptr;     // device parameters of the flip-chain kernels
     int* mc_err_h = nullptr;        // mapped host [2]: a propose kernel gave up waiting; test request
     int* mc_err_d = nullptr;        // its device address
@@ -178,8 +180,8 @@ lrs_status launch_expand_terms(lrs_ctx* ctx, int64_t R, int64_t Rn, cudaStream_t
 // err (may be NULL): per-result bound on |out - exact chi-sum| (see k_amp_reduce).
 lrs_status launch_amplitude(lrs_ctx* ctx, const uint64_t* x, int64_t batch, double* out, float* err,
                             cudaStream_t st);
-lrs_status launch_amplitude_q(lrs_ctx* ctx, const uint64_t* x, int64_t batch, void* Q, double** amp_out,
-                              cudaStream_t st);
+lrs_status launch_amplitude_start(lrs_ctx* ctx, const uint64_t* x, int64_t batch, double** amp_out,
+                                  cudaStream_t st);
 // eta and ov may each be NULL (ov: 2^{n/2} <phi_{A_l}|psi> as Re, Im pairs)
 lrs_status launch_norm_estimate(lrs_ctx* ctx, int64_t L, uint64_t seed, double* eta, double* ov,
                                 cudaStream_t st);
@@ -187,6 +189,9 @@ lrs_status launch_norm_eta(const double* ov, int64_t L, double* eta, cudaStream_
 lrs_status launch_sample_terms(lrs_ctx* ctx, int64_t count, uint64_t seed, uint64_t* x,
                                int64_t* alpha, cudaStream_t st);
 lrs_status launch_chains_init(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st);
+// bytes of the chains' buffers (device memory is the caller's business)
+size_t mc_planes_bytes(const lrs_ctx* ctx);
+size_t mc_state_bytes(const lrs_ctx* ctx, int64_t chains);
 lrs_status launch_metropolis(lrs_ctx* ctx, int64_t steps, uint64_t seed, int64_t step0,
                              uint64_t* x_out, double* p_out, uint64_t* trace, cudaStream_t st);
 lrs_status launch_metropolis_learned(lrs_ctx* ctx, lrs_mlp* mlp, int64_t steps, uint64_t seed,
