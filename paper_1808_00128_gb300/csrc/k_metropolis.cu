@@ -24,8 +24,10 @@
 
 namespace {
 
-constexpr int MC_TPB = 128;    // threads per block
+constexpr int MC_TPB = 256;    // threads per block
+constexpr int MC_COLS = 128;   // most columns of a block
 constexpr int MC_TERMS = 256;  // terms per tile (cap is a multiple of 256)
+constexpr int MC_CG = 32;      // most chains of a block
 
 // ---- bulk-copy helpers (1-D cp.async.bulk completing on an mbarrier) ----------
 constexpr unsigned long long MC_WAIT_NS = 1000000000ull;   // 1 s
@@ -71,19 +73,21 @@ struct McView {
     int64_t cols;
     uint2* J;        // [n (n - 1) / 2 + 1][cols]: J_pq, p > q, row p (p - 1) / 2 + q; the last row zero
     uint2* D;        // [n][2][cols]: d_p, bits 0 and 1
-    uint2* K;        // [n][n][cols]: coefficient of constraint i at qubit p
-    uint2* target;   // [n][cols]: s at constraint i
+    uint4* K;        // [n][pairs][cols]: coefficients of constraints 2 i (x, y) and 2 i + 1 (z, w) at qubit p
+    uint4* target;   // [pairs][cols]: s at the two constraints
+    int pairs;       // (n + 1) / 2
     float2* base;    // [64][cols]: b omega 2^{-|v|/2} / 2 of term (k, l), row 32 k + l (0: no contribution)
     uint8_t* mf;     // [cols / 4]: constraints of the tile (the most of its terms)
 };
 __host__ __device__ __forceinline__ int mc_pairs(int n) { return n * (n - 1) / 2; }
-// Chain states: [plane][chain][cols]: phase bits 0 and 1, the parities J_j1 . x and J_j2 . x of
-// the last pass's proposals, then the constraints' syndromes.
+// Chain states: [plane][chain][cols] of two words, phase bits 0 and 1 and the parities J_j1 . x
+// and J_j2 . x of the last pass's proposals; then [pair][chain][cols] of four, the syndromes
+// of the constraints.
 constexpr int MC_PLANES = 4;
 
 __global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
     extern __shared__ uint64_t sF[];          // [n][256]
-    __shared__ uint32_t sw[2][64][8];         // words of a set of planes for the tile, double-buffered
+    __shared__ uint32_t sw[2][64][16];        // words of a set of planes for the tile, double-buffered
     __shared__ int s_mf;
     const int n = T.n, tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
     const int64_t tile = blockIdx.x, a = tile * MC_TERMS + tid;
@@ -105,10 +109,6 @@ __global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
         V.base[(int64_t)((wi >> 2) * 32 + lane) * V.cols + tile * 4 + (wi & 3)] = b;
     }
     const int64_t row = V.cols * 2;   // words per plane
-    auto flush = [&](uint32_t* dst, int64_t first, int64_t step, int count, int buf) {
-        for (int e = tid; e < count * 8; e += 256)
-            dst[(first + (int64_t)(e >> 3) * step) * row + tile * 8 + (e & 7)] = sw[buf][e >> 3][e & 7];
-    };
     int buf = 0;
     for (int p = 0; p < n; ++p, buf ^= 1) {
         const uint64_t Mp = T.M[(int64_t)p * T.cap + a], Fp = sF[p * 256 + tid];
@@ -124,24 +124,35 @@ __global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
             sw[buf][63][slot] = hi;
         }
         __syncthreads();
-        flush(reinterpret_cast<uint32_t*>(V.J), (int64_t)p * (p - 1) / 2, 1, p, buf);
+        for (int e = tid; e < p * 8; e += 256)
+            reinterpret_cast<uint32_t*>(V.J)[((int64_t)p * (p - 1) / 2 + (e >> 3)) * row + tile * 8 + (e & 7)] =
+                sw[buf][e >> 3][e & 7];
         if (tid < 16)
             reinterpret_cast<uint32_t*>(V.D)[(2 * p + (tid >> 3)) * row + tile * 8 + (tid & 7)] = sw[buf][62 + (tid >> 3)][tid & 7];
     }
     const int mf = s_mf;
     uint64_t ks = out;
-    for (int i = 0; i < mf; ++i, buf ^= 1) {
-        const int k = ks ? ffs64(ks) : -1;   // constraint i of this term: qubit k, or none
+    const int slot4 = (wi & 3) * 4 + (wi >> 2);   // word of this warp in a set of pairs
+    for (int i = 0; 2 * i < mf; ++i, buf ^= 1) {
+        const int k0 = ks ? ffs64(ks) : -1;   // constraint 2 i of this term: qubit k0, or none
         ks &= ks - 1;
-        for (int p = 0; p < n; ++p) {
-            const uint32_t w = __ballot_sync(0xffffffffu, k >= 0 ? (uint32_t)getb(sF[p * 256 + tid], k) : 0u);
-            if (lane == 0) sw[buf][p][slot] = w;
+        const int k1 = ks ? ffs64(ks) : -1;
+        ks &= ks - 1;
+        for (int p = 0; p <= n; ++p) {
+            const uint64_t r = p < n ? sF[p * 256 + tid] : s;   // last: the targets
+            const uint32_t w0 = __ballot_sync(0xffffffffu, k0 >= 0 ? (uint32_t)getb(r, k0) : 0u);
+            const uint32_t w1 = __ballot_sync(0xffffffffu, k1 >= 0 ? (uint32_t)getb(r, k1) : 0u);
+            if (lane == 0) {
+                sw[buf][p][slot4] = w0;
+                sw[buf][p][slot4 + 2] = w1;
+            }
         }
-        const uint32_t tg = __ballot_sync(0xffffffffu, k >= 0 ? (uint32_t)getb(s, k) : 0u);
-        if (lane == 0) sw[buf][63][slot] = tg;
         __syncthreads();
-        flush(reinterpret_cast<uint32_t*>(V.K), (int64_t)i * n, 1, n, buf);
-        if (tid < 8) reinterpret_cast<uint32_t*>(V.target)[i * row + tile * 8 + tid] = sw[buf][63][tid];
+        for (int e = tid; e < (n + 1) * 16; e += 256) {
+            const int p = e >> 4;
+            uint4* dst = p < n ? V.K + ((int64_t)p * V.pairs + i) * V.cols : V.target + (int64_t)i * V.cols;
+            reinterpret_cast<uint32_t*>(dst)[tile * 16 + (e & 15)] = sw[buf][p][e & 15];
+        }
     }
     if (tid == 0) V.mf[tile] = (uint8_t)mf;
     if (tid < 8) reinterpret_cast<uint32_t*>(V.J)[mc_pairs(n) * row + tile * 8 + tid] = 0u;
@@ -149,7 +160,10 @@ __global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
 
 __device__ __forceinline__ uint2 operator^(uint2 a, uint2 b) { return make_uint2(a.x ^ b.x, a.y ^ b.y); }
 __device__ __forceinline__ uint2 operator&(uint2 a, uint2 b) { return make_uint2(a.x & b.x, a.y & b.y); }
-__device__ __forceinline__ uint2 operator|(uint2 a, uint2 b) { return make_uint2(a.x | b.x, a.y | b.y); }
+
+__device__ __forceinline__ uint4 operator^(uint4 a, uint4 b) {
+    return make_uint4(a.x ^ b.x, a.y ^ b.y, a.z ^ b.z, a.w ^ b.w);
+}
 
 // (lo, hi) += +-(dl, dh) + 2 par, in Z4 planes
 __device__ __forceinline__ void z4_step(uint2& lo, uint2& hi, uint2 dl, uint2 dh, bool minus, uint2 par) {
@@ -198,22 +212,23 @@ __global__ void __launch_bounds__(MC_TPB) k_mc_start(McView V, int64_t C, uint2*
     uint2* st = S + c * V.cols + col;
     st[0] = lo;
     st[plane] = hi;
-    const int mf = V.mf[col >> 2];
-    for (int i = 0; i < mf; ++i) {
-        uint2 y = __ldg(V.target + (int64_t)i * V.cols + col);
-        const uint2* Ki = V.K + (int64_t)i * V.n * V.cols + col;
+    uint4* sy = reinterpret_cast<uint4*>(S + MC_PLANES * plane) + c * V.cols + col;
+    const int pairs = (V.mf[col >> 2] + 1) >> 1;
+    for (int i = 0; i < pairs; ++i) {
+        uint4 y = __ldg(V.target + (int64_t)i * V.cols + col);
+        const uint4* Ki = V.K + (int64_t)i * V.cols + col;
         uint64_t r = x;
         while (r) {
-            uint2 t[4];
+            uint4 t[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                t[u] = make_uint2(0u, 0u);
-                if (r) t[u] = __ldg(Ki + (int64_t)ffs64(r) * V.cols);
+                t[u] = make_uint4(0u, 0u, 0u, 0u);
+                if (r) t[u] = __ldg(Ki + (int64_t)ffs64(r) * V.pairs * V.cols);
                 r &= r - 1;
             }
             y = y ^ (t[0] ^ t[1]) ^ (t[2] ^ t[3]);
         }
-        st[(MC_PLANES + i) * plane] = y;
+        sy[i * plane] = y;
     }
 }
 
@@ -231,6 +246,16 @@ __global__ void __launch_bounds__(MC_TPB) k_mc_start(McView V, int64_t C, uint2*
 // At n = 50, chi = 2^20, 256 chains, per step: see the launch below.
 // The block's coefficients (64 rows of tbx columns) are copied once by cp.async.bulk; the wait
 // is bounded (1 s) and a block that gives up sets *err and leaves its sums unwritten.
+// What a pass reads of a chain, gathered once per block: the string, the flips to apply and to
+// propose, and the rows of J at the set bits of x, J_j1q | J_j2q << 16 (rows of zeros for
+// q = j and up to a multiple of eight).
+struct McChain {
+    uint64_t x;
+    int p1, p2, j1, j2;
+    int nq, reserved;
+    uint32_t row[64];
+};
+
 template <int STEPS>
 __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint2* __restrict__ S,
                                                        const uint64_t* __restrict__ cx,
@@ -238,14 +263,16 @@ __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint
                                                        const int32_t* __restrict__ jprop, float2* __restrict__ partial,
                                                        int cg, int64_t groups, int tbx, int* err) {
     constexpr int NE = STEPS == 2 ? 3 : 1;   // strings evaluated
-    extern __shared__ __align__(128) float2 sbase[];   // [64][tbx]
+    extern __shared__ __align__(128) float2 sbase[];   // [64][tbx], then McChain[cg]
     __shared__ __align__(8) uint64_t full;
+    McChain* chains = reinterpret_cast<McChain*>(sbase + 64 * tbx);
     const int tid = threadIdx.x, lane = tid & 31;
     const int64_t c0 = blockIdx.x % groups * cg, tb = blockIdx.x / groups;
     const int nc = (int)(C - c0 < cg ? C - c0 : cg);
     const int nsub = MC_TPB / tbx, tc = tid % tbx;
     const int64_t col0 = tb * tbx;
     const int nb = (int)(V.cols - col0 < tbx ? V.cols - col0 : tbx);   // a multiple of 4
+    const int zero = mc_pairs(V.n);
     const uint32_t bar = mc_smem(&full);
     if (tid == 0) {
         mc_bar_init(bar);
@@ -261,6 +288,28 @@ __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint
         for (int r = 0; r < 64; ++r)
             mc_bulk_load(mc_smem(sbase + r * tbx), V.base + (int64_t)r * V.cols + col0, (uint32_t)(nb * sizeof(float2)), bar);
     }
+    for (int ci = tid >> 5; ci < nc; ci += MC_TPB / 32) {   // a warp per chain
+        McChain& ch = chains[ci];
+        const int64_t c = c0 + ci;
+        const uint64_t x = cx[c];
+        const int j1 = jprop[c], j2 = STEPS == 2 ? jprop[C + c] : 0, nq = __popcll(x);
+        if (lane == 0) {
+            ch.x = x;
+            ch.p1 = pend[c];
+            ch.p2 = pend[C + c];
+            ch.j1 = j1;
+            ch.j2 = j2;
+            ch.nq = nq;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int q = lane + 32 * h;
+            if (getb(x, q))
+                ch.row[__popcll(x & (bit64(q) - 1))] =
+                    (uint32_t)mc_row(j1, q, zero) | (uint32_t)(STEPS == 2 ? mc_row(j2, q, zero) : zero) << 16;
+        }
+        if (lane < ((8 - nq) & 7)) ch.row[nq + lane] = (uint32_t)zero | (uint32_t)zero << 16;
+    }
     __syncthreads();
     if (__syncthreads_or(!mc_bar_wait(bar, 0u))) {
         // every copy has landed or is waited for once more (bounded) before the block leaves
@@ -272,164 +321,167 @@ __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint
     }
     const bool in = tc < nb;
     const int64_t col = col0 + (in ? tc : 0), plane = C * V.cols, n_tiles = V.cols >> 2;
-    const int mf = V.mf[col >> 2];
-    const int mfw = __reduce_max_sync(0xffffffffu, mf);
-    const int zero = mc_pairs(V.n);
-    const uint2* J = V.J + col;
-    const uint2* D = V.D + col;
+    const int mf2 = (V.mf[col >> 2] + 1) >> 1;   // pairs of constraints of the tile
+    const int mfw = __reduce_max_sync(0xffffffffu, mf2);
+    const uint32_t row8 = (uint32_t)V.cols * 8u;   // bytes of a plane (cols <= 2^28)
+    const char* Jc = reinterpret_cast<const char*>(V.J + col);
+    const char* Dc = reinterpret_cast<const char*>(V.D + col);
+    auto J = [&](uint32_t r) { return __ldg(reinterpret_cast<const uint2*>(Jc + (uint64_t)r * row8)); };
+    auto D = [&](uint32_t r) { return __ldg(reinterpret_cast<const uint2*>(Dc + (uint64_t)r * row8)); };
     const float2* bp = sbase + tc;
     const uint2 none = make_uint2(0u, 0u);
     for (int i0 = 0; i0 < nc; i0 += nsub) {
-        const int ci = i0 + tid / tbx;
-        const bool on = in && ci < nc;
-        const int64_t c = c0 + (ci < nc ? ci : 0);
-        const uint64_t x = cx[c];
-        const int p1 = pend[c], p2 = pend[C + c], j1 = jprop[c], j2 = STEPS == 2 ? jprop[C + c] : 0;
+        const int ci = i0 + tid / tbx < nc ? i0 + tid / tbx : 0;
+        const bool on = in && i0 + tid / tbx < nc;
+        const McChain& ch = chains[ci];
+        const int64_t c = c0 + ci;
+        const uint64_t x = ch.x;
+        const int p1 = ch.p1, p2 = ch.p2, j1 = ch.j1, j2 = ch.j2;
         uint2* st = S + c * V.cols + col;
         uint2 lo = st[0], hi = st[plane];
         const bool moved = p1 >= 0 || p2 >= 0;
+        uint2 old1 = none, old2 = none;
+        if (p1 >= 0) old1 = st[2 * plane];
+        if (p2 >= 0) old2 = st[3 * plane];
+        // J_j . x for the proposals
+        uint2 par1 = none, par2 = none;
+#pragma unroll 1
+        for (int k = 0; k < ch.nq; k += 8) {
+            uint2 t1[8], t2[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const uint32_t r = ch.row[k + u];
+                t1[u] = J(r & 0xffffu);
+                if (STEPS == 2) t2[u] = J(r >> 16);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; u += 2) {
+                par1 = par1 ^ t1[u] ^ t1[u + 1];
+                if (STEPS == 2) par2 = par2 ^ t2[u] ^ t2[u + 1];
+            }
+        }
         if (moved) {   // the flips accepted after the previous pass, in order
             uint64_t xo = x ^ (p1 >= 0 ? bit64(p1) : 0ull) ^ (p2 >= 0 ? bit64(p2) : 0ull);
-            uint2 par2 = p2 >= 0 ? st[3 * plane] : none;
             if (p1 >= 0) {
-                z4_step(lo, hi, __ldg(D + (int64_t)(2 * p1) * V.cols), __ldg(D + (int64_t)(2 * p1 + 1) * V.cols), getb(xo, p1) != 0,
-                        st[2 * plane]);
+                z4_step(lo, hi, D(2 * p1), D(2 * p1 + 1), getb(xo, p1) != 0, old1);
                 xo ^= bit64(p1);
-                if (p2 >= 0) par2 = par2 ^ __ldg(J + (int64_t)mc_row(p1, p2, zero) * V.cols);
+                if (p2 >= 0) old2 = old2 ^ J(mc_row(p1, p2, zero));
             }
-            if (p2 >= 0)
-                z4_step(lo, hi, __ldg(D + (int64_t)(2 * p2) * V.cols), __ldg(D + (int64_t)(2 * p2 + 1) * V.cols), getb(xo, p2) != 0,
-                        par2);
+            if (p2 >= 0) z4_step(lo, hi, D(2 * p2), D(2 * p2 + 1), getb(xo, p2) != 0, old2);
             if (on) {
                 st[0] = lo;
                 st[plane] = hi;
             }
         }
-        // J_j . x for the proposals (the zero row stands in for q = j and past the last bit)
-        uint2 par1 = none, par2 = none;
-        for (uint64_t r = x; r;) {
-            uint2 t1[4], t2[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int q = r ? ffs64(r) : j1;
-                t1[u] = __ldg(J + (int64_t)mc_row(j1, q, zero) * V.cols);
-                if (STEPS == 2) t2[u] = __ldg(J + (int64_t)(r ? mc_row(j2, q, zero) : zero) * V.cols);
-                r &= r - 1;
-            }
-            par1 = par1 ^ (t1[0] ^ t1[1]) ^ (t1[2] ^ t1[3]);
-            if (STEPS == 2) par2 = par2 ^ (t2[0] ^ t2[1]) ^ (t2[2] ^ t2[3]);
-        }
         if (on) {
             st[2 * plane] = par1;
             if (STEPS == 2) st[3 * plane] = par2;
         }
-        // phases of y1, y1 ^ e_j2, x ^ e_j2
+        // phases of y1, y1 ^ e_j2, x ^ e_j2 and the terms whose constraints fail there
         uint2 L[NE], H[NE], dead[NE];
-        {
-            const uint2 dl = __ldg(D + (int64_t)(2 * j1) * V.cols), dh = __ldg(D + (int64_t)(2 * j1 + 1) * V.cols);
-            L[0] = lo;
-            H[0] = hi;
-            z4_step(L[0], H[0], dl, dh, getb(x, j1) != 0, par1);
-            dead[0] = none;
-        }
+        L[0] = lo;
+        H[0] = hi;
+        z4_step(L[0], H[0], D(2 * j1), D(2 * j1 + 1), getb(x, j1) != 0, par1);
         if (STEPS == 2) {
-            const uint2 dl = __ldg(D + (int64_t)(2 * j2) * V.cols), dh = __ldg(D + (int64_t)(2 * j2 + 1) * V.cols);
-            const uint2 j12 = __ldg(J + (int64_t)mc_row(j1, j2, zero) * V.cols);
-            L[1] = L[0];
-            H[1] = H[0];
-            z4_step(L[1], H[1], dl, dh, getb(x ^ bit64(j1), j2) != 0, par2 ^ j12);
+            const uint2 dl = D(2 * j2), dh = D(2 * j2 + 1), j12 = J(mc_row(j1, j2, zero));
+            L[NE / 2] = L[0];
+            H[NE / 2] = H[0];
+            z4_step(L[NE / 2], H[NE / 2], dl, dh, getb(x ^ bit64(j1), j2) != 0, par2 ^ j12);
             L[NE - 1] = lo;
             H[NE - 1] = hi;
             z4_step(L[NE - 1], H[NE - 1], dl, dh, getb(x, j2) != 0, par2);
-            dead[1] = none;
-            dead[NE - 1] = none;
         }
-#pragma unroll 2
-        for (int i = 0; i < mfw; ++i) {
-            if (i >= mf) continue;   // this tile has fewer
-            const uint2* Ki = V.K + (int64_t)i * V.n * V.cols + col;
-            uint2 y = st[(MC_PLANES + i) * plane];
-            const uint2 k1 = __ldg(Ki + (int64_t)j1 * V.cols), k2 = STEPS == 2 ? __ldg(Ki + (int64_t)j2 * V.cols) : none;
-            if (moved) {
-                if (p1 >= 0) y = y ^ __ldg(Ki + (int64_t)p1 * V.cols);
-                if (p2 >= 0) y = y ^ __ldg(Ki + (int64_t)p2 * V.cols);
-                if (on) st[(MC_PLANES + i) * plane] = y;
-            }
-            dead[0] = dead[0] | (y ^ k1);
-            if (STEPS == 2) {
-                dead[1] = dead[1] | (y ^ k1 ^ k2);
-                dead[NE - 1] = dead[NE - 1] | (y ^ k2);
-            }
-        }
-        // sums
-        bool some = false;
 #pragma unroll
-        for (int e = 0; e < NE; ++e) some = some || (dead[e].x & dead[e].y) != 0xffffffffu;
-        float2 f[NE], u[NE];
-#pragma unroll
-        for (int e = 0; e < NE; ++e) f[e] = u[e] = make_float2(0.f, 0.f);
-        if (__any_sync(0xffffffffu, some)) {
+        for (int e = 0; e < NE; ++e) dead[e] = none;
+        uint4* sy = reinterpret_cast<uint4*>(S + MC_PLANES * plane) + c * V.cols + col;
+        const uint4* K = V.K + col;
+        const int64_t krow = (int64_t)V.pairs * V.cols;
 #pragma unroll 1
-            for (int it = 0; it < 4; ++it) {
-                // leaves l = l0 + 4 t, l0 = bits 0 and 1 of l
-                const int l0 = (it >> 1) + 2 * (it & 1);
-                uint32_t N0[NE], N1[NE];   // nibble t: live, phase bit 1, phase bit 0
-#pragma unroll
-                for (int e = 0; e < NE; ++e) {
+        for (int i = 0; i < mfw; ++i, K += V.cols, sy += plane) {
+            if (i >= mf2) continue;   // this tile has fewer
+            uint4 y = *sy;
+            const uint4 k1 = __ldg(K + j1 * krow);
+            uint4 k2;
+            if (STEPS == 2) k2 = __ldg(K + j2 * krow);
+            if (moved) {
+                if (p1 >= 0) y = y ^ __ldg(K + p1 * krow);
+                if (p2 >= 0) y = y ^ __ldg(K + p2 * krow);
+                if (on) *sy = y;
+            }
+            const uint4 y1 = y ^ k1;
+            dead[0].x |= y1.x | y1.z;
+            dead[0].y |= y1.y | y1.w;
+            if (STEPS == 2) {
+                dead[NE / 2].x |= (y1.x ^ k2.x) | (y1.z ^ k2.z);
+                dead[NE / 2].y |= (y1.y ^ k2.y) | (y1.w ^ k2.w);
+                dead[NE - 1].x |= (y.x ^ k2.x) | (y.z ^ k2.z);
+                dead[NE - 1].y |= (y.y ^ k2.y) | (y.w ^ k2.w);
+            }
+        }
+        // the sums, one string at a time (rolled: registers for three blocks an SM)
+#pragma unroll 1
+        for (int e = 0; e < NE; ++e) {
+            float2 f = make_float2(0.f, 0.f), u = f;
+            if (__any_sync(0xffffffffu, (dead[0].x & dead[0].y) != 0xffffffffu)) {
+#pragma unroll 1
+                for (int it = 0; it < 4; ++it) {
+                    // leaves l = l0 + 4 t, l0 = bits 0 and 1 of l; nibble t of N: live, phase
+                    // bit 1, phase bit 0
+                    const int l0 = (it >> 1) + 2 * (it & 1);
                     constexpr uint32_t one = 0x11111111u;
-                    N0[e] = (~dead[e].x >> l0 & one) | (H[e].x >> l0 & one) << 1 | (L[e].x >> l0 & one) << 2;
-                    N1[e] = (~dead[e].y >> l0 & one) | (H[e].y >> l0 & one) << 1 | (L[e].y >> l0 & one) << 2;
-                }
-                const float2* b0 = bp + l0 * tbx;
-                float2 v[NE][8];
+                    const uint32_t N0 =
+                        (~dead[0].x >> l0 & one) | (H[0].x >> l0 & one) << 1 | (L[0].x >> l0 & one) << 2;
+                    const uint32_t N1 =
+                        (~dead[0].y >> l0 & one) | (H[0].y >> l0 & one) << 1 | (L[0].y >> l0 & one) << 2;
+                    const float2* b0 = bp + l0 * tbx;
+                    float2 v[8];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const float2 ba = b0[4 * t * tbx], bb = b0[(32 + 4 * t) * tbx];
-#pragma unroll
-                    for (int e = 0; e < NE; ++e) {
+                    for (int t = 0; t < 8; ++t) {
+                        const float2 ba = b0[4 * t * tbx], bb = b0[(32 + 4 * t) * tbx];
                         // b i^m, m = 2 hi + lo: (x, y) or (-y, x), times (-1)^hi
-                        const float fa = __uint_as_float((N0[e] << (30 - 4 * t)) & 0xC0000000u);
-                        const float fb = __uint_as_float((N1[e] << (30 - 4 * t)) & 0xC0000000u);
-                        const bool sa = (N0[e] & (4u << (4 * t))) != 0, sb = (N1[e] & (4u << (4 * t))) != 0;
-                        const float rx = fa * (sa ? -ba.y : ba.x), ry = fa * (sa ? ba.x : ba.y);
-                        v[e][t].x = fmaf(fb, sb ? -bb.y : bb.x, rx);
-                        v[e][t].y = fmaf(fb, sb ? bb.x : bb.y, ry);
+                        const float fa = __uint_as_float((N0 << (30 - 4 * t)) & 0xC0000000u);
+                        const float fb = __uint_as_float((N1 << (30 - 4 * t)) & 0xC0000000u);
+                        const bool sa = (N0 & (4u << (4 * t))) != 0, sb = (N1 & (4u << (4 * t))) != 0;
+                        v[t].x = fmaf(fb, sb ? -bb.y : bb.x, fa * (sa ? -ba.y : ba.x));
+                        v[t].y = fmaf(fb, sb ? bb.x : bb.y, fa * (sa ? ba.x : ba.y));
                     }
-                }
-#pragma unroll
-                for (int e = 0; e < NE; ++e) {
 #pragma unroll
                     for (int h = 4; h > 0; h >>= 1)   // bits 4, 3, 2 of l
 #pragma unroll
                         for (int t = 0; t < h; ++t) {
-                            v[e][t].x += v[e][t + h].x;
-                            v[e][t].y += v[e][t + h].y;
+                            v[t].x += v[t + h].x;
+                            v[t].y += v[t + h].y;
                         }
                     // bit 1, then bit 0
                     if (it & 1) {
-                        u[e].x += v[e][0].x;
-                        u[e].y += v[e][0].y;
+                        u.x += v[0].x;
+                        u.y += v[0].y;
                     } else {
-                        u[e] = v[e][0];
+                        u = v[0];
                     }
-                    if (it == 1) f[e] = u[e];
+                    if (it == 1) f = u;
                     if (it == 3) {
-                        f[e].x += u[e].x;
-                        f[e].y += u[e].y;
+                        f.x += u.x;
+                        f.y += u.y;
                     }
                 }
             }
-        }
-        // the four columns of the tile in order
-#pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            float2 acc = f[e];
+            // the four columns of the tile in order
+            float2 acc = f;
 #pragma unroll
             for (int w = 1; w < 4; ++w) {
-                acc.x += __shfl_down_sync(0xffffffffu, f[e].x, w);
-                acc.y += __shfl_down_sync(0xffffffffu, f[e].y, w);
+                acc.x += __shfl_down_sync(0xffffffffu, f.x, w);
+                acc.y += __shfl_down_sync(0xffffffffu, f.y, w);
             }
             if (on && (lane & 3) == 0) partial[((int64_t)e * C + c) * n_tiles + (col >> 2)] = acc;
+            if (NE == 3) {   // next string
+                L[0] = L[NE / 2];
+                H[0] = H[NE / 2];
+                dead[0] = dead[NE / 2];
+                L[NE / 2] = L[NE - 1];
+                H[NE / 2] = H[NE - 1];
+                dead[NE / 2] = dead[NE - 1];
+            }
         }
     }
 }
@@ -683,8 +735,9 @@ static size_t mc_layout(const lrs_ctx* ctx, McView* V) {
     v.base = (float2*)take(64);
     v.J = (uint2*)take(mc_pairs(n) + 1);
     v.D = (uint2*)take(2 * n);
-    v.K = (uint2*)take((size_t)n * n);
-    v.target = (uint2*)take(n);
+    v.pairs = (n + 1) / 2;
+    v.K = (uint4*)take((size_t)2 * n * v.pairs);
+    v.target = (uint4*)take((size_t)2 * v.pairs);
     v.mf = (uint8_t*)take(1);   // cols / 4 bytes
     if (V) *V = v;
     return at;
@@ -692,13 +745,13 @@ static size_t mc_layout(const lrs_ctx* ctx, McView* V) {
 
 size_t mc_planes_bytes(const lrs_ctx* ctx) { return mc_layout(ctx, nullptr); }
 size_t mc_state_bytes(const lrs_ctx* ctx, int64_t chains) {
-    return (size_t)(MC_PLANES + ctx->n) * chains * (ctx->cap / 64) * sizeof(uint2);
+    return (size_t)(MC_PLANES + 2 * ((ctx->n + 1) / 2)) * chains * (ctx->cap / 64) * sizeof(uint2);
 }
 
 // Columns per block: 128, fewer (a power of two) for a context of fewer terms, whose
 // blocks then take several chains at a time.
 static int mc_columns(int64_t cols) {
-    int t = MC_TPB;
+    int t = MC_COLS;
     while (t > 4 && t / 2 >= cols) t /= 2;
     return t;
 }
@@ -741,15 +794,17 @@ static lrs_status mc_pass(lrs_ctx* ctx, int steps, const int32_t* jprop, float2*
     const int64_t C = ctx->n_chains;
     const int tbx = mc_columns(V.cols), nsub = MC_TPB / tbx;
     const int64_t tblocks = (V.cols + tbx - 1) / tbx;
-    // chains per block: up to the tuned number, fewer while the grid is under four
-    // rounds of three blocks per SM (a block's coefficients are one copy of 64 KB)
+    // chains per block: up to the tuned number and what leaves room for three blocks per
+    // SM, fewer while the grid is under four rounds of them (a block's coefficients are
+    // one copy of 64 KB)
     const int64_t want = ((int64_t)12 * ctx->sm_count + tblocks - 1) / tblocks;
     int64_t cg = (C + want - 1) / want;
     if (cg < nsub) cg = nsub;
     if (cg > ctx->tune_mc_cg) cg = ctx->tune_mc_cg;
+    if (cg > MC_CG) cg = MC_CG;
     const int64_t groups = (C + cg - 1) / cg, blocks = tblocks * groups;
     if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "Metropolis grid too large");
-    const size_t smem = (size_t)64 * tbx * sizeof(float2);
+    const size_t smem = (size_t)64 * tbx * sizeof(float2) + cg * sizeof(McChain);
     if (steps == 2)
         k_mc_pass<2><<<(unsigned)blocks, MC_TPB, smem, st>>>(V, C, (uint2*)ctx->Q, ctx->cx, ctx->pend, jprop, partial,
                                                              (int)cg, groups, tbx, ctx->mc_err_d);
@@ -763,7 +818,7 @@ static lrs_status mc_pass(lrs_ctx* ctx, int steps, const int32_t* jprop, float2*
 static lrs_status mc_attributes(cudaStream_t st) {
     // inside a graph capture the attributes were set by an earlier uncaptured call
     if (lrs_capturing(st)) return LRS_OK;
-    const int most = (int)(64 * MC_TPB * sizeof(float2));
+    const int most = (int)(64 * MC_COLS * sizeof(float2) + MC_CG * sizeof(McChain));
     LRS_CUDA(cudaFuncSetAttribute(k_mc_pass<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     LRS_CUDA(cudaFuncSetAttribute(k_mc_pass<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     return LRS_OK;
