@@ -317,6 +317,308 @@ __global__ void k_amp_reduce_batch(const __grid_constant__ AmpBatch B, int64_t t
     }
 }
 
+// ---- bit-sliced amplitudes -------------------------------------------------------------
+// <x|phi> = b omega 2^{-|v|/2} i^{q(x)} where F_k . x = s_k for every k not in v (F_k: column k
+// of F), else 0, with the Z4 form
+//     q(x) = sum_p d_p x_p + 2 sum_{p<q} J_pq x_p x_q,   J = M F^T,
+//     d_p = gamma_p + 2 F_p . M_p + 2 F_p . (s & v),
+// or, with sum_p lo_p x_p = P + 2 sum_{p<q} lo_p lo_q x_p x_q (P its parity, lo_p = d_p mod 2),
+//     q(x) = P + 2 (hi . x + sum_p x_p (L_p . x)),   L_p = (J_pq + lo_p lo_q) over q < p.
+// k_amp_prep writes lo, hi, the rows L_p and the constraints of every term once (a warp per
+// term); k_amp_sliced evaluates these linear forms on 32 strings at a time, bit i of a word
+// belonging to string i: a form is the XOR, over chunks of six qubits, of one entry of a
+// table of the chunk's 64 XORs of string words, which depends on the strings only
+// and serves every term.  Per (term, 1024 strings) that is about n^2 / 12 + 1.5 n + n / 6 per
+// constraint shared-memory loads of 128 bytes and three integer instructions each, where one
+// string per thread takes 8 ceil(n / 4) + 16 instructions for 32 strings.
+constexpr int AS_WARPS = 8, AS_TPB = 32 * AS_WARPS;
+constexpr int AS_CB = 6;       // qubits per chunk
+constexpr int AS_TERMS = 32;   // terms whose words the block collects before summing
+enum { AMP_INFO = 0, AMP_VAL, AMP_LO, AMP_HI, AMP_ROWS };   // record: header, rows L_0.., constraints
+
+struct AmpPrep {
+    uint64_t* rec;   // [terms][words]
+    int words, rows; // rows = chunks * AS_CB
+};
+
+// Records of terms [a0, a0 + count): a warp per term, lane c holding rows c and c + 32.
+__global__ void __launch_bounds__(256) k_amp_prep(TermsView T, int64_t a0, int64_t count, AmpPrep P) {
+    __shared__ uint64_t sF[8][64];
+    const int n = T.n, lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), a = a0 + i;
+    if (i >= count) return;
+    const uint64_t v = T.v[a], s = T.s[a], glo = T.glo[a], ghi = T.ghi[a];
+    const uint32_t om = T.omega[a];
+    uint64_t* rec = P.rec + i * P.words;
+    const bool live = ((om >> 3) & 1u) == 0u;
+    const uint64_t out = ~v & T.nmask;
+    const int mf = __popcll(out);
+    if (lane == 0) {
+        const float2 b = T.coef[a];
+        const int e0 = __popcll(v) + (int)(om >> 8);
+        const float2 val = z8_scale(b, (int)(om & 7u), e0);
+        const float mag = ldexpf(hypotf(b.x, b.y), -(e0 >> 1)) * ((e0 & 1) ? 0.70710678f : 1.f);
+        rec[AMP_INFO] = (uint64_t)((uint32_t)mf | (live ? 1u << 8 : 0u)) | (uint64_t)__float_as_uint(mag) << 32;
+        rec[AMP_VAL] = (uint64_t)__float_as_uint(val.x) | (uint64_t)__float_as_uint(val.y) << 32;
+    }
+    if (!live) return;
+    uint64_t F[2], M[2], J[2] = {0, 0};
+    uint32_t hi[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int q = lane + 32 * c;
+        F[c] = q < n ? T.F[(int64_t)q * T.cap + a] : 0ull;
+        M[c] = q < n ? T.M[(int64_t)q * T.cap + a] : 0ull;
+        hi[c] = (uint32_t)getb(ghi, q) ^ par64(F[c] & M[c]) ^ par64(F[c] & s & v);
+    }
+    uint64_t* rows = sF[threadIdx.x >> 5];
+    rows[lane] = F[0];
+    rows[lane + 32] = F[1];
+    __syncwarp();
+    lrs_products(rows, n, M[0], M[1], J[0], J[1]);
+    const uint64_t hw = (uint64_t)__ballot_sync(0xffffffffu, hi[0]) | (uint64_t)__ballot_sync(0xffffffffu, hi[1]) << 32;
+    if (lane == 0) {
+        rec[AMP_LO] = glo;
+        rec[AMP_HI] = hw & T.nmask;
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int p = lane + 32 * c;
+        if (p < P.rows) rec[AMP_ROWS + p] = p < n ? (J[c] ^ (getb(glo, p) ? glo : 0ull)) & (bit64(p) - 1) : 0ull;
+    }
+    // constraints: the columns of F outside v
+    uint64_t ks = out;
+    for (int k = 0; k < mf; ++k) {
+        const int q = ffs64(ks);
+        ks &= ks - 1;
+        const uint64_t col = (uint64_t)__ballot_sync(0xffffffffu, (uint32_t)getb(F[0], q)) |
+                             (uint64_t)__ballot_sync(0xffffffffu, (uint32_t)getb(F[1], q)) << 32;
+        if (lane == 0) rec[AMP_ROWS + P.rows + k] = col;
+    }
+    if (lane == 0) {
+        rec[AMP_ROWS + P.rows + n] = s;       // targets: s_k of the k-th qubit outside v
+        rec[AMP_ROWS + P.rows + n + 1] = v;
+    }
+}
+
+// Linear form w over the first NC chunks: XOR of table entries of this lane's column.  `tab` is the
+// shared address of the lane's column; the table starts on an 8 KB boundary, so that
+// masking the pattern (times 128 bytes) out of the word and adding the address is one
+// three-input operation.
+template <int C>
+__device__ __forceinline__ uint32_t amp_entry(uint32_t tab, uint32_t lo, uint32_t hi) {
+    constexpr int sh = AS_CB * C - 7;
+    uint32_t t, a, r;
+    if (sh < 0)
+        t = lo << (sh < 0 ? -sh : 0);
+    else if (sh < 32)
+        t = __funnelshift_r(lo, hi, sh >= 0 ? sh : 0);
+    else
+        t = hi >> (sh >= 32 ? sh - 32 : 0);
+    asm("lop3.b32 %0, %1, 0x1f80, %2, 0xea;" : "=r"(a) : "r"(t), "r"(tab));   // (t & 0x1f80) | tab
+    asm("ld.shared.u32 %0, [%1 + %2];" : "=r"(r) : "r"(a), "n"(C * 64 * 128));
+    return r;
+}
+template <int NC, int C = 0>
+__device__ __forceinline__ uint32_t amp_form(uint32_t tab, uint64_t w) {
+    const uint32_t lo = (uint32_t)w, hi = (uint32_t)(w >> 32);
+    if constexpr (C + 2 < NC)
+        return amp_entry<C>(tab, lo, hi) ^ amp_entry<C + 1>(tab, lo, hi) ^ amp_form<NC, C + 2>(tab, w);
+    else if constexpr (C + 2 == NC)
+        return amp_entry<C>(tab, lo, hi) ^ amp_entry<C + 1>(tab, lo, hi);
+    else
+        return amp_entry<C>(tab, lo, hi);
+}
+template <int P>   // the string words of qubit P
+__device__ __forceinline__ uint32_t amp_bit(uint32_t tab) {
+    uint32_t r;
+    asm("ld.shared.u32 %0, [%1 + %2];" : "=r"(r) : "r"(tab), "n"((P / AS_CB * 64 + (1 << P % AS_CB)) * 128));
+    return r;
+}
+
+// Rows p = C AS_CB .. of the quadratic part: sum over p of x_p (L_p . x), chunk row by chunk
+// row, the next chunk's rows loaded while this one's are evaluated.
+struct AmpRows {
+    ulonglong2 r[AS_CB / 2];
+};
+__device__ __forceinline__ AmpRows amp_load(const ulonglong2* __restrict__ rows, int c) {
+    AmpRows R;
+#pragma unroll
+    for (int i = 0; i < AS_CB / 2; ++i) R.r[i] = __ldg(rows + c * (AS_CB / 2) + i);
+    return R;
+}
+template <int NC, int C>
+__device__ __forceinline__ void amp_rows(uint32_t tab, const ulonglong2* __restrict__ rows, const AmpRows& cur, int n,
+                                         uint32_t& acc) {
+    AmpRows next = cur;
+    if constexpr (C + 1 < NC) next = amp_load(rows, C + 1);
+    constexpr int P = C * AS_CB;
+    if (P > 0) acc ^= amp_form<C + 1>(tab, cur.r[0].x) & amp_bit<P>(tab);
+    if (C + 1 < NC || P + 1 < n) acc ^= amp_form<C + 1>(tab, cur.r[0].y) & amp_bit<P + 1>(tab);
+    if (C + 1 < NC || P + 2 < n) {
+        acc ^= amp_form<C + 1>(tab, cur.r[1].x) & amp_bit<P + 2>(tab);
+        acc ^= amp_form<C + 1>(tab, cur.r[1].y) & amp_bit<P + 3>(tab);
+    }
+    if (C + 1 < NC || P + 4 < n) {
+        acc ^= amp_form<C + 1>(tab, cur.r[2].x) & amp_bit<P + 4>(tab);
+        acc ^= amp_form<C + 1>(tab, cur.r[2].y) & amp_bit<P + 5>(tab);
+    }
+    if constexpr (C + 1 < NC) amp_rows<NC, C + 1>(tab, rows, next, n, acc);
+}
+
+// Kahan sum of the complex pair s with the negated compensation nc, both parts at once (the
+// operations of KahanC::add, packed), where `on` is not zero.
+__device__ __forceinline__ void kahan_add2(uint64_t& s, uint64_t& nc, float x, float y, uint32_t on) {
+    asm("{\n"
+        " .reg .pred p;\n .reg .b64 a, t, d, m;\n"
+        " setp.ne.u32 p, %4, 0;\n"
+        " mov.b64 a, {%2, %3};\n"
+        " mov.b64 m, {%5, %5};\n"
+        " add.rn.f32x2 a, a, %1;\n"        // x - c
+        " add.rn.f32x2 t, %0, a;\n"
+        " fma.rn.f32x2 d, t, m, %0;\n"     // s - t
+        " @p add.rn.f32x2 %1, a, d;\n"     // -((t - s) - (x - c))
+        " @p mov.b64 %0, t;\n"
+        "}"
+        : "+l"(s), "+l"(nc)
+        : "f"(x), "f"(y), "r"(on), "f"(-1.f));
+}
+
+// A block: 8 warps, G = 32 / wl term tiles (wl string words of 32 strings each, a power of
+// two: 32 for 1024 strings and one tile).  Lane (g, l) = (lane / wl, lane % wl) holds
+// word l for tile g.  The warps first evaluate AS_TERMS terms of every tile, one term each at
+// a time, leaving three words per lane and term (live, phase bits); then thread (warp, lane)
+// adds up the four strings 4 warp .. 4 warp + 3 of its lane's word, in term order, so every
+// string's Kahan sum over a tile is the one a single thread would form.
+// The table takes 8 KB per chunk (72 KB at n = 50): two blocks an SM.
+template <int NC, bool ERR>
+__global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint64_t nmask, const uint64_t* __restrict__ xs,
+                                                          int64_t batch, int64_t tt, int64_t cap, int64_t a0, int64_t tile0,
+                                                          int64_t tile1, int64_t n_tiles, int wl, int64_t tgroups,
+                                                          float2* __restrict__ partial, float* __restrict__ magp) {
+    // shared memory: table (on an 8 KB boundary), then the collected words and values, whose
+    // place holds the string words while the table is built
+    extern __shared__ __align__(16) unsigned char dyn[];
+    const uint32_t dyn0 = (uint32_t)__cvta_generic_to_shared(dyn);
+    const uint32_t tab0 = (dyn0 + 8191u) & ~8191u;
+    uint32_t* tabw = reinterpret_cast<uint32_t*>(dyn + (tab0 - dyn0));                             // [NC][64][32]
+    uint32_t(*sw)[3][32] = reinterpret_cast<uint32_t(*)[3][32]>(tabw + NC * 64 * 32);              // live, phase bits
+    uint32_t(*sx)[32] = &sw[0][0];                                                                 // [NC AS_CB][32]
+    float2(*sval)[32] = reinterpret_cast<float2(*)[32]>(&sw[AS_TERMS][0][0]);                      // [AS_TERMS][32]
+    float(*smag)[32] = reinterpret_cast<float(*)[32]>(&sval[AS_TERMS][0]);                         // [AS_TERMS][32] (ERR)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t tg = blockIdx.x % tgroups, xb = blockIdx.x / tgroups;
+    const int G = 32 / wl, g = lane / wl, l = lane % wl;
+    // string words: warp per word, ballots over its 32 strings
+    for (int w = warp; w < wl; w += AS_WARPS) {
+        const int64_t i = (xb * wl + w) * 32 + lane;
+        const uint64_t x = i < batch ? xs[i] & nmask : 0ull;
+        for (int p = 0; p < NC * AS_CB; ++p) {
+            const uint32_t b = __ballot_sync(0xffffffffu, p < 64 && ((x >> (p & 63)) & 1ull) != 0);
+            if (lane < G) sx[p][lane * wl + w] = b;
+        }
+    }
+    __syncthreads();
+    for (int c = warp; c < NC; c += AS_WARPS) {
+        uint32_t* t = tabw + c * 64 * 32 + lane;
+        uint32_t cur = 0;
+        t[0] = 0;
+#pragma unroll
+        for (int k = 1; k < 64; ++k) {   // Gray code: one XOR an entry
+            const int bit = __ffs(k) - 1;
+            cur ^= sx[c * AS_CB + bit][lane];
+            t[(k ^ (k >> 1)) * 32] = cur;
+        }
+    }
+    __syncthreads();
+    const int64_t tile = tile0 + tg * G + g;
+    const int64_t b0 = tile < tile1 ? tile * tt : 0;
+    const int64_t len = tile < tile1 ? (b0 + tt < cap ? tt : cap - b0) : 0;   // of this lane's tile
+    uint32_t tl;   // opaque and after the barrier: the table's loads depend on it
+    asm volatile("add.u32 %0, %1, %2;" : "=r"(tl) : "r"(tab0), "r"(4u * lane) : "memory");
+    uint64_t sum[4], nc[4];   // complex pairs
+    float mag[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        sum[k] = nc[k] = 0;
+        mag[k] = 0.f;
+    }
+    for (int64_t c0 = 0; c0 < tt; c0 += AS_TERMS) {
+#pragma unroll 1
+        for (int t = warp; t < AS_TERMS && c0 + t < tt; t += AS_WARPS) {
+            const bool have = c0 + t < len;
+            const uint64_t* rec = P.rec + (have ? b0 + c0 + t - a0 : 0) * P.words;
+            const ulonglong2 head = __ldg(reinterpret_cast<const ulonglong2*>(rec));
+            const ulonglong2 lin = __ldg(reinterpret_cast<const ulonglong2*>(rec + AMP_LO));
+            const bool on = have && ((uint32_t)head.x >> 8 & 1u);
+            {   // the warp's next record on its way
+                const char* nx = reinterpret_cast<const char*>(rec + (int64_t)AS_WARPS * P.words) + l * 128;
+                if (c0 + t + AS_WARPS < len && l * 16 < AMP_ROWS + P.rows)
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(nx));
+            }
+            const int mf = on ? (int)(head.x & 255u) : 0;
+            uint32_t live = on ? 0xffffffffu : 0u;
+            const uint64_t* cons = rec + AMP_ROWS + P.rows;
+            const uint64_t tgt = mf > 0 ? __ldg(cons + n) : 0ull;
+            uint64_t ks = mf > 0 ? ~__ldg(cons + n + 1) & nmask : 0ull;
+            const int most = __reduce_max_sync(0xffffffffu, mf);
+#pragma unroll 1
+            for (int k = 0; k < most; ++k) {
+                if (k < mf) {
+                    const uint32_t y = amp_form<NC>(tl, __ldg(cons + k));
+                    const uint32_t want = 0u - (uint32_t)((tgt & ks & (0ull - ks)) != 0);
+                    ks &= ks - 1;
+                    live &= ~(y ^ want);
+                }
+                if (!__any_sync(0xffffffffu, live != 0u)) break;
+            }
+            uint32_t ph0 = 0, ph1 = 0;
+            if (__any_sync(0xffffffffu, live != 0u)) {
+                ph0 = amp_form<NC>(tl, lin.x);
+                ph1 = amp_form<NC>(tl, lin.y);
+                const ulonglong2* rows = reinterpret_cast<const ulonglong2*>(rec + AMP_ROWS);
+                amp_rows<NC, 0>(tl, rows, amp_load(rows, 0), n, ph1);
+            }
+            sw[t][0][lane] = live;
+            sw[t][1][lane] = ph0;
+            sw[t][2][lane] = ph1;
+            if (l == 0) {
+                sval[t][g] = make_float2(__uint_as_float((uint32_t)head.y), __uint_as_float((uint32_t)(head.y >> 32)));
+                if (ERR) smag[t][g] = __uint_as_float((uint32_t)(head.x >> 32));
+            }
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int t = 0; t < AS_TERMS && c0 + t < tt; ++t) {
+            const uint32_t live = sw[t][0][lane] >> (4 * warp) & 15u;
+            if (!__any_sync(0xffffffffu, live != 0u)) continue;
+            const uint32_t q0 = sw[t][1][lane] >> (4 * warp), q1 = sw[t][2][lane] >> (4 * warp);
+            const float2 b = sval[t][g];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool odd = (q0 >> k) & 1u;   // i^m b, m = q0 + 2 q1
+                const uint32_t neg = (q1 << (31 - k)) & 0x80000000u;
+                const uint32_t rx = __float_as_uint(odd ? -b.y : b.x), ry = __float_as_uint(odd ? b.x : b.y);
+                kahan_add2(sum[k], nc[k], __uint_as_float(rx ^ neg), __uint_as_float(ry ^ neg), live & (1u << k));
+                if (ERR && (live >> k & 1u)) mag[k] += smag[t][g];
+            }
+        }
+        __syncthreads();
+    }
+    if (tile < tile1) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t i = (xb * wl + l) * 32 + 4 * warp + k;
+            if (i < batch) {
+                partial[i * n_tiles + tile] =
+                    make_float2(__uint_as_float((uint32_t)sum[k]) + __uint_as_float((uint32_t)nc[k]),
+                                __uint_as_float((uint32_t)(sum[k] >> 32)) + __uint_as_float((uint32_t)(nc[k] >> 32)));
+                if (ERR) magp[i * n_tiles + tile] = mag[k];
+            }
+        }
+    }
+}
+
 struct AmpPlan {
     int64_t xblocks, n_tiles, tt;
 };
@@ -353,6 +655,73 @@ lrs_status launch_amp_t(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* 
     return LRS_OK;
 }
 
+template <int NC>
+lrs_status launch_sliced_t(lrs_ctx* ctx, const AmpPrep& R, const uint64_t* x, int64_t batch, const AmpPlan& P, int64_t a0,
+                           int64_t tile0, int64_t tile1, int wl, float2* partial, float* magp, cudaStream_t st) {
+    // up to 8 KB to the table's boundary, the table, the collected words and values
+    const size_t smem = 8192 + (size_t)NC * 8192 +
+                        (size_t)AS_TERMS * 32 * (3 * sizeof(uint32_t) + sizeof(float2) + (magp ? sizeof(float) : 0));
+    const auto kernel = magp ? k_amp_sliced<NC, true> : k_amp_sliced<NC, false>;
+    if (!lrs_capturing(st))
+        LRS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int64_t G = 32 / wl, tgroups = (tile1 - tile0 + G - 1) / G;
+    const int64_t blocks = tgroups * ((batch + 32 * wl - 1) / (32 * wl));
+    if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "amplitude grid too large");
+    kernel<<<(unsigned)blocks, AS_TPB, smem, st>>>(R, ctx->n, ctx->nmask, x, batch, P.tt, ctx->cap, a0, tile0, tile1,
+                                                   P.n_tiles, wl, tgroups, partial, magp);
+    LRS_LAUNCH_CHECK("amplitude kernel");
+    return LRS_OK;
+}
+
+// Tile sums of the batch by the sliced kernel, the records of at most AMP_REC_BYTES of terms
+// at a time in `rec`.
+constexpr size_t AMP_REC_BYTES = (size_t)512 << 20;
+AmpPrep amp_records(const lrs_ctx* ctx) {
+    AmpPrep R;
+    R.rec = nullptr;
+    R.rows = (ctx->n + AS_CB - 1) / AS_CB * AS_CB;
+    R.words = (AMP_ROWS + R.rows + ctx->n + 2 + 15) & ~15;   // lines of 128 bytes
+    return R;
+}
+// tiles whose records are held at a time
+int64_t amp_tiles_at_once(const AmpPrep& R, const AmpPlan& P) {
+    int64_t t = (int64_t)(AMP_REC_BYTES / ((size_t)P.tt * R.words * sizeof(uint64_t)));
+    if (t < 32) t = 32;   // a block may take 32 tiles
+    t &= ~(int64_t)31;
+    return t < P.n_tiles ? t : P.n_tiles;
+}
+
+lrs_status launch_sliced(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* partial, const AmpPlan& P, AmpPrep R,
+                         float* magp, cudaStream_t st) {
+    // string words of a block: 32 (1024 strings), fewer for a batch that has fewer, whose
+    // blocks then take several tiles
+    int wl = 32;
+    while (wl > 1 && batch <= 16 * wl) wl /= 2;
+    const int64_t step = amp_tiles_at_once(R, P);
+    for (int64_t t0 = 0; t0 < P.n_tiles; t0 += step) {
+        const int64_t t1 = t0 + step < P.n_tiles ? t0 + step : P.n_tiles;
+        const int64_t a0 = t0 * P.tt, a1 = t1 * P.tt < ctx->cap ? t1 * P.tt : ctx->cap;
+        k_amp_prep<<<(unsigned)((a1 - a0 + 7) / 8), 256, 0, st>>>(ctx->view(), a0, a1 - a0, R);
+        LRS_LAUNCH_CHECK("amplitude prep kernel");
+        lrs_status rc;
+        switch (R.rows / AS_CB) {
+            case 1: rc = launch_sliced_t<1>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 2: rc = launch_sliced_t<2>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 3: rc = launch_sliced_t<3>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 4: rc = launch_sliced_t<4>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 5: rc = launch_sliced_t<5>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 6: rc = launch_sliced_t<6>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 7: rc = launch_sliced_t<7>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 8: rc = launch_sliced_t<8>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 9: rc = launch_sliced_t<9>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 10: rc = launch_sliced_t<10>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            default: rc = launch_sliced_t<11>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+        }
+        if (rc != LRS_OK) return rc;
+    }
+    return LRS_OK;
+}
+
 lrs_status launch_amp_kernels(lrs_ctx* ctx, const uint64_t* x, int64_t batch, double* out,
                               float2* partial, const AmpPlan& P, cudaStream_t st,
                               float* magp = nullptr, float* err = nullptr) {
@@ -384,29 +753,50 @@ lrs_status launch_amp_kernels(lrs_ctx* ctx, const uint64_t* x, int64_t batch, do
 
 }  // namespace
 
+// The sliced kernels and the reduction, with scratch for partial sums, bounds (err), amplitudes
+// (*amp_out) and records; the string-per-thread kernel where the records do not fit.
+static lrs_status launch_amp_scratch(lrs_ctx* ctx, const uint64_t* x, int64_t batch, const AmpPlan& P, double* out,
+                                     double** amp_out, float* err, cudaStream_t st) {
+    const size_t part = ((size_t)batch * P.n_tiles * sizeof(float2) + 255) & ~(size_t)255;
+    const size_t mags = err ? ((size_t)batch * P.n_tiles * sizeof(float) + 255) & ~(size_t)255 : 0;
+    const size_t amps = amp_out ? ((size_t)batch * 2 * sizeof(double) + 255) & ~(size_t)255 : 0;
+    AmpPrep R = amp_records(ctx);
+    int64_t terms = amp_tiles_at_once(R, P) * P.tt;
+    if (terms > ctx->cap) terms = ctx->cap;
+    const size_t need = part + mags + amps;
+    void* scr = nullptr;
+    lrs_status rc = lrs_scratch(ctx, need + (size_t)terms * R.words * sizeof(uint64_t), &scr);
+    const bool sliced = rc == LRS_OK;
+    if (rc == LRS_ERR_OOM) {
+        cudaGetLastError();   // the failed allocation's error is not the next launch's
+        rc = lrs_scratch(ctx, need, &scr);
+    }
+    if (rc != LRS_OK) return rc;
+    float2* partial = (float2*)scr;
+    float* magp = err ? (float*)((char*)scr + part) : nullptr;
+    if (amp_out) out = *amp_out = (double*)((char*)scr + part + mags);
+    if (!sliced) return launch_amp_kernels(ctx, x, batch, out, partial, P, st, magp, err);
+    R.rec = (uint64_t*)((char*)scr + need);
+    if ((rc = launch_sliced(ctx, x, batch, partial, P, R, magp, st)) != LRS_OK) return rc;
+    k_amp_reduce<<<(unsigned)batch, 256, 0, st>>>(partial, magp, P.n_tiles, batch, P.tt, out, err);
+    LRS_LAUNCH_CHECK("amplitude reduce kernel");
+    return LRS_OK;
+}
+
 // Amplitudes of the chains' start strings into scratch (*amp_out, 2 doubles per x), on the
 // term tiles of 512 strings per block.
 lrs_status launch_amplitude_start(lrs_ctx* ctx, const uint64_t* x, int64_t batch, double** amp_out, cudaStream_t st) {
     AmpPlan P = amp_plan(ctx, batch, 512);
     P.xblocks = (batch + AMP_XB - 1) / AMP_XB;
-    const size_t part = ((size_t)batch * P.n_tiles * sizeof(float2) + 255) & ~(size_t)255;
-    void* scr = nullptr;
-    lrs_status rc = lrs_scratch(ctx, part + (size_t)batch * 2 * sizeof(double), &scr);
-    if (rc != LRS_OK) return rc;
-    *amp_out = (double*)((char*)scr + part);
-    return launch_amp_kernels(ctx, x, batch, *amp_out, (float2*)scr, P, st);
+    return launch_amp_scratch(ctx, x, batch, P, nullptr, amp_out, nullptr, st);
 }
 
 lrs_status launch_amplitude(lrs_ctx* ctx, const uint64_t* x, int64_t batch, double* out, float* err,
                             cudaStream_t st) {
     if (batch == 0) return LRS_OK;
     const AmpPlan P = amp_plan(ctx, batch, AMP_XB);
-    const size_t part = ((size_t)batch * P.n_tiles * sizeof(float2) + 255) & ~(size_t)255;
-    void* scr = nullptr;
-    lrs_status rc = lrs_scratch(ctx, part + (err ? (size_t)batch * P.n_tiles * sizeof(float) : 0), &scr);
-    if (rc != LRS_OK) return rc;
-    float* magp = err ? (float*)((char*)scr + part) : nullptr;
-    return launch_amp_kernels(ctx, x, batch, out, (float2*)scr, P, st, magp, err);
+    if (P.xblocks > 65535) return lrs_fail(LRS_ERR_UNSUPPORTED, "amplitude batch too large");
+    return launch_amp_scratch(ctx, x, batch, P, out, nullptr, err, st);
 }
 
 template <int NCH>
@@ -425,6 +815,18 @@ static lrs_status launch_amp_batch_t(const AmpBatch& B, int64_t blocks, bool pk,
 lrs_status launch_amplitude_batch(lrs_ctx* const* ctxs, const uint64_t* const* xs, const int64_t* batch,
                                   double* const* out, int32_t count, cudaStream_t st) {
     const int n = ctxs[0]->n;
+    // Large circuits one after the other by the sliced kernel (each fills the GPU); small
+    // ones, where its launches per circuit would add up, together.  The line: 2^23 (x, term)
+    // per circuit take about 60 us either way.
+    double work = 0.0;
+    for (int32_t i = 0; i < count; ++i) work += (double)ctxs[i]->cap * (double)batch[i];
+    if (work >= (double)count * 8388608.0) {
+        for (int32_t i = 0; i < count; ++i) {
+            const lrs_status rc = launch_amplitude(ctxs[i], xs[i], batch[i], out[i], nullptr, st);
+            if (rc != LRS_OK) return rc;
+        }
+        return LRS_OK;
+    }
     for (int32_t base = 0; base < count; base += LRS_AMP_BATCH_MAX) {
         AmpBatch B;
         memset(&B, 0, sizeof(B));

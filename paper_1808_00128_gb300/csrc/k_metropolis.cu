@@ -246,6 +246,12 @@ __global__ void __launch_bounds__(MC_TPB) k_mc_start(McView V, int64_t C, uint2*
 // At n = 50, chi = 2^20, 256 chains, per step: see the launch below.
 // The block's coefficients (64 rows of tbx columns) are copied once by cp.async.bulk; the wait
 // is bounded (1 s) and a block that gives up sets *err and leaves its sums unwritten.
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {   // two FP32 additions
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // What a pass reads of a chain, gathered once per block: the string, the flips to apply and to
 // propose, and the rows of J at the set bits of x, J_j1q | J_j2q << 16 (rows of zeros for
 // q = j and up to a multiple of eight).
@@ -421,7 +427,7 @@ __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint
         // the sums, one string at a time (rolled: registers for three blocks an SM)
 #pragma unroll 1
         for (int e = 0; e < NE; ++e) {
-            float2 f = make_float2(0.f, 0.f), u = f;
+            uint64_t f2 = 0, u = 0;
             if (__any_sync(0xffffffffu, (dead[0].x & dead[0].y) != 0xffffffffu)) {
 #pragma unroll 1
                 for (int it = 0; it < 4; ++it) {
@@ -434,7 +440,7 @@ __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint
                     const uint32_t N1 =
                         (~dead[0].y >> l0 & one) | (H[0].y >> l0 & one) << 1 | (L[0].y >> l0 & one) << 2;
                     const float2* b0 = bp + l0 * tbx;
-                    float2 v[8];
+                    uint64_t v[8];   // complex pairs
 #pragma unroll
                     for (int t = 0; t < 8; ++t) {
                         const float2 ba = b0[4 * t * tbx], bb = b0[(32 + 4 * t) * tbx];
@@ -442,31 +448,22 @@ __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint
                         const float fa = __uint_as_float((N0 << (30 - 4 * t)) & 0xC0000000u);
                         const float fb = __uint_as_float((N1 << (30 - 4 * t)) & 0xC0000000u);
                         const bool sa = (N0 & (4u << (4 * t))) != 0, sb = (N1 & (4u << (4 * t))) != 0;
-                        v[t].x = fmaf(fb, sb ? -bb.y : bb.x, fa * (sa ? -ba.y : ba.x));
-                        v[t].y = fmaf(fb, sb ? bb.x : bb.y, fa * (sa ? ba.x : ba.y));
+                        const float re = fmaf(fb, sb ? -bb.y : bb.x, fa * (sa ? -ba.y : ba.x));
+                        const float im = fmaf(fb, sb ? bb.x : bb.y, fa * (sa ? ba.x : ba.y));
+                        asm("mov.b64 %0, {%1, %2};" : "=l"(v[t]) : "f"(re), "f"(im));
                     }
 #pragma unroll
                     for (int h = 4; h > 0; h >>= 1)   // bits 4, 3, 2 of l
 #pragma unroll
-                        for (int t = 0; t < h; ++t) {
-                            v[t].x += v[t + h].x;
-                            v[t].y += v[t + h].y;
-                        }
+                        for (int t = 0; t < h; ++t) v[t] = add2(v[t], v[t + h]);
                     // bit 1, then bit 0
-                    if (it & 1) {
-                        u.x += v[0].x;
-                        u.y += v[0].y;
-                    } else {
-                        u = v[0];
-                    }
-                    if (it == 1) f = u;
-                    if (it == 3) {
-                        f.x += u.x;
-                        f.y += u.y;
-                    }
+                    u = (it & 1) ? add2(u, v[0]) : v[0];
+                    if (it == 1) f2 = u;
+                    if (it == 3) f2 = add2(f2, u);
                 }
             }
             // the four columns of the tile in order
+            const float2 f = make_float2(__uint_as_float((uint32_t)f2), __uint_as_float((uint32_t)(f2 >> 32)));
             float2 acc = f;
 #pragma unroll
             for (int w = 1; w < 4; ++w) {
@@ -486,26 +483,37 @@ __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint
     }
 }
 
+// |sum over tiles|^2 of chain c in FP64, by each group of 256 threads; valid in the group's
+// first warp's lane 0.  (The last five levels of the tree by shuffles: same pairs.)
 __device__ __forceinline__ double chain_reduce(const float2* __restrict__ partial, int64_t c,
                                                int64_t n_tiles) {
+    const int tid = threadIdx.x & 255;
     double re = 0.0, im = 0.0;
-    for (int64_t t = threadIdx.x; t < n_tiles; t += blockDim.x) {
+    for (int64_t t = tid; t < n_tiles; t += 256) {
         const float2 p = partial[c * n_tiles + t];
         re += (double)p.x;
         im += (double)p.y;
     }
-    __shared__ double sre[256], sim[256];
+    __shared__ double sre[768], sim[768];
     sre[threadIdx.x] = re;
     sim[threadIdx.x] = im;
     __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if ((int)threadIdx.x < off) {
+    for (int off = 128; off >= 64; off >>= 1) {
+        if (tid < off) {
             sre[threadIdx.x] += sre[threadIdx.x + off];
             sim[threadIdx.x] += sim[threadIdx.x + off];
         }
         __syncthreads();
     }
-    return sre[0] * sre[0] + sim[0] * sim[0];
+    if (tid >= 32) return 0.0;
+    re = sre[threadIdx.x] + sre[threadIdx.x + 32];
+    im = sim[threadIdx.x] + sim[threadIdx.x + 32];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        re += __shfl_down_sync(0xffffffffu, re, off);
+        im += __shfl_down_sync(0xffffffffu, im, off);
+    }
+    return re * re + im * im;
 }
 
 __device__ __forceinline__ int draw_j(uint64_t seed, int64_t c, int64_t step, int n) {
@@ -577,12 +585,15 @@ __global__ void k_metro_accept(const float2* __restrict__ partial, int64_t n_til
 __global__ void k_metro_accept2(const float2* __restrict__ partial, int64_t n_tiles,
                                 const McParams* __restrict__ P, int64_t t, int n, uint64_t* cx, double* cp,
                                 int32_t* pend, int32_t* jprop, uint64_t* trace, int64_t C) {
+    // the three sums, by as many groups of 256 threads as the block has (three or one)
+    __shared__ double prob[3];
     const int64_t c = blockIdx.x;
-    const double p1 = chain_reduce(partial, c, n_tiles);
-    __syncthreads();   // every thread has read the first result before the shared sums are reused
-    const double p2a = chain_reduce(partial + C * n_tiles, c, n_tiles);
-    __syncthreads();
-    const double p2r = chain_reduce(partial + 2 * C * n_tiles, c, n_tiles);
+    for (int r = threadIdx.x >> 8; r < 3; r += blockDim.x >> 8) {
+        const double pr = chain_reduce(partial + r * C * n_tiles, c, n_tiles);
+        if ((threadIdx.x & 255) == 0) prob[r] = pr;
+        __syncthreads();
+    }
+    const double p1 = prob[0], p2a = prob[1], p2r = prob[2];
     if (threadIdx.x == 0) {
         const uint64_t seed = P->seed;
         const uint64_t key = sm64_key(seed, (uint64_t)c);
@@ -834,7 +845,7 @@ static lrs_status enqueue_steps(lrs_ctx* ctx, int64_t t0, int64_t count, float2*
     if (ctx->tune_mc_lookahead == 2) {
         for (; t + 1 < t0 + count; t += 2) {
             if ((rc = mc_pass(ctx, 2, jprop, partial, st)) != LRS_OK) return rc;
-            k_metro_accept2<<<(unsigned)C, 256, 0, st>>>(partial, n_tiles, ctx->mc_par, t, ctx->n, ctx->cx,
+            k_metro_accept2<<<(unsigned)C, n_tiles >= 1024 ? 768 : 256, 0, st>>>(partial, n_tiles, ctx->mc_par, t, ctx->n, ctx->cx,
                                                           ctx->cp, ctx->pend, jprop,
                                                           trace ? trace + t * C : nullptr, C);
             LRS_LAUNCH_CHECK("metropolis two-step accept kernel");

@@ -118,6 +118,7 @@ __device__ __forceinline__ uint64_t drop_bits(uint64_t x, uint64_t keep, uint64_
 }
 
 __global__ void __launch_bounds__(256) k_norm_prep(TermsView T, NormPrep P) {
+    __shared__ uint64_t sF[8][64];
     const int n = T.n, lane = threadIdx.x & 31;
     const int64_t alpha = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (alpha >= T.chi) return;   // warp-uniform; padding terms need no record
@@ -133,11 +134,11 @@ __global__ void __launch_bounds__(256) k_norm_prep(TermsView T, NormPrep P) {
         // diagonal of q_J + 2 (F s) . y' (Z4)
         d[c] = (uint32_t)getb(glo, q) | ((uint32_t)getb(ghi, q) ^ par64(F[c] & s)) << 1;
     }
-    for (int e = 0; e < n; ++e) {
-        const uint64_t Fe = shfl64(e < 32 ? F[0] : F[1], e & 31);
-        J[0] |= (uint64_t)par64(M[0] & Fe) << e;
-        J[1] |= (uint64_t)par64(M[1] & Fe) << e;
-    }
+    uint64_t* rows = sF[threadIdx.x >> 5];
+    rows[lane] = F[0];
+    rows[lane + 32] = F[1];
+    __syncwarp();
+    lrs_products(rows, n, M[0], M[1], J[0], J[1]);
 #pragma unroll
     for (int c = 0; c < 2; ++c) J[c] &= ~bit64(lane + 32 * c);
     // constraint i in lane i % 32: column k_i of F (k_i the i-th qubit outside v) and s_{k_i}

@@ -35,6 +35,30 @@ __device__ __forceinline__ int ffs64(uint64_t x) {  // index of lowest set bit, 
 __device__ __forceinline__ uint64_t bit64(int j) { return 1ull << j; }
 __device__ __forceinline__ uint64_t getb(uint64_t x, int j) { return (x >> j) & 1ull; }
 
+// Bit e of J0, J1 = parity(M0 & row e), parity(M1 & row e), e < n: two rows of M F^T per lane,
+// rows[] = F in shared memory (the same address for all lanes).  A parity's bit is shifted
+// in from the top with one funnel shift.
+__device__ __forceinline__ void lrs_products(const uint64_t* rows, int n, uint64_t M0, uint64_t M1, uint64_t& J0,
+                                             uint64_t& J1) {
+    uint32_t w[2][2] = {{0u, 0u}, {0u, 0u}};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int e1 = n < 32 * h + 32 ? n : 32 * h + 32;
+#pragma unroll 4
+        for (int e = 32 * h; e < e1; ++e) {
+            const uint64_t F = rows[e];
+            w[0][h] = __funnelshift_r(w[0][h], __popc((uint32_t)(M0 & F) ^ (uint32_t)((M0 & F) >> 32)), 1);
+            w[1][h] = __funnelshift_r(w[1][h], __popc((uint32_t)(M1 & F) ^ (uint32_t)((M1 & F) >> 32)), 1);
+        }
+        const int rest = 32 * h + 32 - e1;   // bits not shifted in
+        if (rest > 0)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) w[r][h] = rest < 32 ? w[r][h] >> rest : 0u;
+    }
+    J0 = w[0][0] | (uint64_t)w[0][1] << 32;
+    J1 = w[1][0] | (uint64_t)w[1][1] << 32;
+}
+
 // ---- exact Z8 phase times power of sqrt2, rounded once to FP32 -------------------
 // returns b * exp(i pi ph / 4) * 2^(-e/2)  (ph any int, e any int)
 __device__ __forceinline__ float2 z8_scale(float2 b, int ph, int e) {
