@@ -11,6 +11,11 @@
 namespace {
 
 // ---- init_terms: one thread per term ---------------------------------------------
+// FP64 units are what the sparsified draw is short of (about 16 cycles of an SM per warp
+// instruction), so a draw is compared as a 53-bit integer with the cumulative
+// probabilities scaled by 2^53 (u < cdf exactly), and the product of the phases skips
+// the factors that are exactly 1 (every first choice of an RZ slot), in slot order, so the
+// product's roundings are the same.
 __global__ void k_init_terms(TermsView T, int32_t mode, uint64_t seed, double scale) {
     const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= T.cap) return;
@@ -46,20 +51,30 @@ __global__ void k_init_terms(TermsView T, int32_t mode, uint64_t seed, double sc
     } else {
         bre = scale; bim = 0.0;
         const uint64_t key = sm64_key(seed, (uint64_t)(T.alpha0 + a));
-        for (int64_t p = 0; p < T.n_slots; ++p) {
-            const DevSlot& S = T.slots[p];
-            const double u = sm64_unit(sm64_at(key, (uint64_t)p));
-            int j = -1, last = 0;
-            for (int c = 0; c < S.n_choices; ++c) {
-                if (S.c_re[c] == 0.0 && S.c_im[c] == 0.0) continue;
-                last = c;
-                if (j < 0 && u < S.cdf[c]) j = c;
+        for (int64_t p0 = 0; p0 < T.n_slots; p0 += 64) {   // 64 slots' choices, then their phases
+            const int64_t p1 = p0 + 64 < T.n_slots ? p0 + 64 : T.n_slots;
+            uint64_t turn = 0;
+            for (int64_t p = p0; p < p1; ++p) {
+                const DevSlot& S = T.slots[p];
+                const uint64_t u = sm64_at(key, (uint64_t)p) >> 11;
+                int j = -1, last = 0;
+                for (int c = 0; c < S.n_choices; ++c) {
+                    if (!(S.nonzero >> c & 1)) continue;
+                    last = c;
+                    if (j < 0 && u < S.cdf53[c]) j = c;
+                }
+                if (j < 0) j = last;
+                T.choice[p * T.cap + a] = (uint8_t)j;
+                if (!(S.one >> j & 1)) turn |= 1ull << (p - p0);
             }
-            if (j < 0) j = last;
-            T.choice[p * T.cap + a] = (uint8_t)j;
-            const double xr = bre * S.ph_re[j] - bim * S.ph_im[j];
-            const double xi = bre * S.ph_im[j] + bim * S.ph_re[j];
-            bre = xr; bim = xi;
+            for (; turn; turn &= turn - 1) {
+                const int64_t p = p0 + ffs64(turn);
+                const DevSlot& S = T.slots[p];
+                const int j = T.choice[p * T.cap + a];
+                const double xr = bre * S.ph_re[j] - bim * S.ph_im[j];
+                const double xi = bre * S.ph_im[j] + bim * S.ph_re[j];
+                bre = xr; bim = xi;
+            }
         }
     }
     T.coef[a] = make_float2((float)bre, (float)bim);

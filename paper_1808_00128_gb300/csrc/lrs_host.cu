@@ -443,16 +443,20 @@ extern "C" lrs_status lrs_init_terms(lrs_ctx* c, const lrs_slot* slots, int64_t 
             d.c_re[j] = s.c_re[j];
             d.c_im[j] = s.c_im[j];
             norm += hypot(s.c_re[j], s.c_im[j]);
-            if (s.c_re[j] != 0.0 || s.c_im[j] != 0.0) d.nz_idx[d.n_nonzero++] = j;
+            if (s.c_re[j] != 0.0 || s.c_im[j] != 0.0) {
+                d.nz_idx[d.n_nonzero++] = j;
+                d.nonzero |= 1 << j;
+            }
         }
         if (d.n_nonzero == 0) return lrs_fail(LRS_ERR_ARG, "slot %lld: all coefficients zero", (long long)p);
         double acc = 0.0;
         for (int j = 0; j < s.n_choices; ++j) {
             const double a = hypot(s.c_re[j], s.c_im[j]);
             acc += a / norm;
-            d.cdf[j] = acc;
+            d.cdf53[j] = (uint64_t)ceil(acc * 9007199254740992.0);   // u 2^53 < acc 2^53, u 2^53 whole
             d.ph_re[j] = a > 0 ? s.c_re[j] / a : 0.0;
             d.ph_im[j] = a > 0 ? s.c_im[j] / a : 0.0;
+            if (d.ph_re[j] == 1.0 && d.ph_im[j] == 0.0) d.one |= 1 << j;
         }
         l1 *= norm;
         exact_chi *= d.n_nonzero;

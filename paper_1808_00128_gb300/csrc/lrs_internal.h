@@ -29,7 +29,8 @@ struct DevSlot {
     int32_t nz_idx[LRS_MAX_CHOICES];   // nonzero choices in index order
     int32_t k_off[LRS_MAX_CHOICES];
     int32_t k_len[LRS_MAX_CHOICES];
-    double cdf[LRS_MAX_CHOICES];       // cumulative |c_j| / ||c||_1 (sparsify)
+    int32_t one, nonzero;              // bit j: c_j / |c_j| is exactly 1; c_j is not zero
+    uint64_t cdf53[LRS_MAX_CHOICES];   // cumulative |c_j| / ||c||_1 times 2^53, rounded up (sparsify)
     double c_re[LRS_MAX_CHOICES], c_im[LRS_MAX_CHOICES];     // c_j (exact)
     double ph_re[LRS_MAX_CHOICES], ph_im[LRS_MAX_CHOICES];   // c_j / |c_j| (sparsify)
 };
