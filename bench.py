@@ -68,7 +68,7 @@ def parse(argv=None):
     ap.add_argument("--config5-graph", action="store_true",
                     help="only config 5's eight-circuit step, uncaptured and as one CUDA graph")
     ap.add_argument("--hs-sum8-chains", action="store_true",
-                    help="only the chains on the 2^24-term hidden shift (1024 chains, 206 GB of Pauli states)")
+                    help="only the chains on the 2^24-term hidden shift (1024 chains, their bit-plane states)")
     ap.add_argument("--qaoa-apply-only", action="store_true",
                     help="run only apply_clifford on the n=50 QAOA circuit at chi = 2^16, twice, and "
                          "print its times (for ncu captures; not a bench line)")
@@ -169,14 +169,71 @@ def metropolis_bytes(chi, C, T, n, accept=0.5, lookahead=1):
     return (T // 2) * two + (T % 2) * one
 
 
+def amplitude_sliced_ops_per_unit(n, vw):
+    """32-bit integer ops per (x, term) of the bit-sliced kernel: three per table entry of
+    32 strings (rows p of the quadratic part: p // 6 + 1 chunks and the qubit's own word;
+    two linear forms and one per constraint: ceil(n / 6) each), and eight per string for the
+    live bit, the swap and the sign of a term's value."""
+    import numpy as np
+    chunks = (n + 5) // 6
+    entries = sum(p // 6 + 2 for p in range(n)) + chunks * (2 + float(np.mean(n - np.asarray(vw))))
+    return 3.0 * entries / 32.0 + 8.0
+
+
+def norm_sliced_ops_per_unit(n, vw):
+    """32-bit integer ops per (A, term) of the bit-sliced kernel (instructions of a warp per 32
+    equatorial states, one per state): per pair of variables two per entry of the rows
+    left, 64 columns above 32 variables and 32 below, and the partner search (8 rows); two
+    per entry and constraint, two per entry to form and lift the rows; 60 per variable left to
+    the per-state end (10)."""
+    import numpy as np
+    total = []
+    for m in np.asarray(vw):
+        m = int(m)
+        cols = 2 if m > 32 else 1
+        ops = cols * m * (4.25 + 4 * (n - m)) + 60 * min(m, 10)
+        r = m
+        while r > 10:
+            c = 2 if r > 32 else 1
+            ops += 2 * c * (r - 2) + 8 * (4 + c)
+            r -= 2
+        total.append(ops)
+    return np.array(total, dtype=float)
+
+
+def metropolis_plane_bytes(chi, C, T, n, mf, accept=0.5, lookahead=1):
+    """HBM bytes of T steps on bit-planes: per (chain, 64 terms) and pass 8-byte words, two phase
+    planes read, two parity planes written, mf syndromes read (mf: constraints of a
+    256-term tile), and after an accepted move two parities read and phases and syndromes
+    written; the terms' planes (J, constraints, d) and coefficients once per pass."""
+    moved = 1 - (1 - accept) ** lookahead
+    words = 2 + 2 + mf + moved * (2 + 2 + mf)
+    planes = n * (n - 1) / 2 + n * mf + 2 * n
+    passes = T // lookahead + T % lookahead
+    return passes * (C * chi / 64 * 8 * words + chi * (planes / 8 + 8))
+
+
+def record_launches(n, chi, B, per_block, sms=152, blocks_per_sm=8):
+    """Launches of the amplitude records and sums (two per 512 MB of records)."""
+    cap = (chi + 255) // 256 * 256
+    xblocks = (B + per_block - 1) // per_block
+    nt = max(1, min((sms * blocks_per_sm + xblocks - 1) // xblocks, (cap + 31) // 32))
+    tt = ((cap + nt - 1) // nt + 7) // 8 * 8
+    tiles = (cap + tt - 1) // tt
+    words = (4 + (n + 5) // 6 * 6 + n + 2 + 15) // 16 * 16
+    step = max(32, (512 << 20) // (tt * words * 8)) // 32 * 32
+    return 2 * ((tiles + step - 1) // step)
+
+
 def units_per_step(chi, B, C, T):
     return chi * (B + C * (T + 1))
 
 
 def launches_per_step(T, lookahead=1):
-    """Library kernels one step launches: init, apply, amplitude + reduce, norm (prep,
-    equatorial draws, norm, reduce), chain starts, chains_init (amplitude with Pauli
-    states, reduce, chain scalars), Metropolis (set, first, graphs of 16 steps with
+    """Library kernels one step launches, with one launch for the sums of an amplitude batch
+    (record_launches counts the actual ones): init, apply, amplitude + reduce, norm (prep,
+    equatorial draws, norm, reduce), chain starts, chains_init (amplitude, reduce, chain
+    scalars; its plane and state kernels come on top), Metropolis (set, first, graphs of 16 steps with
     2 launches per pass of `lookahead` steps and an advance node, the remaining steps,
     out)."""
     g, r = divmod(T, 16)
@@ -189,8 +246,8 @@ def launches_per_step(T, lookahead=1):
 # dram__bytes_write.sum), per unit of work, with the hash of the kernel source the
 # capture ran; `traffic` is reported only while that source is unchanged.
 TRAFFIC = {
-    # k_norm<13, 7> on the profiling case (n = 50 QAOA, chi = 2^16, L = 64): 34,172,672 B
-    # read + 185,088 B written per launch for 2^16 x 64 (A, term) units
+    # a form-per-thread k_norm on the profiling case (n = 50 QAOA, chi = 2^16, L = 64):
+    # 34,172,672 B read + 185,088 B written per launch for 2^16 x 64 (A, term) units
     "norm_estimate": {"bytes_per_unit": (34172672 + 185088) / (65536 * 64),
                       "source": "paper_1808_00128_gb300/csrc/k_norm.cu", "sha16": "8f42b33d2b5067dc",
                       "profile": "profiles/k_norm_n50_chi65536_L64.md"},
@@ -457,7 +514,7 @@ class StepRunner:
 
     @property
     def lookahead(self):
-        """Metropolis steps per pass over the Pauli states (the context's knob, read
+        """Metropolis steps per pass over the chain states (the context's knob, read
         while the context is open and kept)."""
         if getattr(self, "_look", None) is None:
             self._look = self.sim.get_tuning("mc_lookahead")
@@ -536,6 +593,12 @@ class StepRunner:
         d2h = amp_h.numel() * 8 + eta_h.numel() * 8 + xo_h.numel() * 8 + po_h.numel() * 8
         return statistics.mean(ms), h2d, d2h
 
+    def launches(self):
+        """Library kernels one step launches."""
+        s = self.shape
+        return (launches_per_step(s["T"], self.lookahead) + record_launches(self.n, self.chi, s["B"], 1024) - 1
+                + 2 + record_launches(self.n, self.chi, s["C"], 512) - 1)
+
     def rooflines(self, phase_ms, alu_peak, hbm_peak):
         """Per phase: achieved and fraction of the roofline on the kernel's own op count
         and on the hot-path table's formula."""
@@ -545,12 +608,12 @@ class StepRunner:
         vw = np.array([bin(int(v)).count("1") for v in ex["v"]])
         xs = self.x_host.numpy().view(np.uint64)
         xpop = float(np.mean([bin(int(x)).count("1") for x in xs]))
-        folds = self.sim.get_tuning("norm_max_folds")
+        tile_mf = float(np.mean([(n - vw[i:i + 256]).max() for i in range(0, len(vw), 256)]))
         ops = {
             "apply_clifford": (chi * clifford_ops_per_term(n, self.low), chi * clifford_ops_per_term(n, self.low, True)),
-            "amplitude": (chi * s["B"] * amplitude_ops_per_unit(n, xpop),
+            "amplitude": (chi * s["B"] * amplitude_sliced_ops_per_unit(n, vw),
                           chi * s["B"] * amplitude_ops_per_unit(n, xpop, True)),
-            "norm_estimate": (chi * s["L"] * float(np.mean(norm_ops_per_unit(n, vw, folds))),
+            "norm_estimate": (chi * s["L"] * float(np.mean(norm_sliced_ops_per_unit(n, vw))),
                               chi * s["L"] * float(np.mean(norm_ops_per_unit(n, vw, -1)))),
         }
         units = {"apply_clifford": ("term-gates", chi * len(self.low.gates)),
@@ -563,9 +626,9 @@ class StepRunner:
                        "frac": k_ops / t / alu_peak, "frac_formula": f_ops / t / alu_peak, "ms": phase_ms[p],
                        "rate": units[p][1] / t, "rate_unit": units[p][0] + "/s"}
         t = phase_ms["metropolis"] * 1e-3
-        # the kernel's own bytes (two steps per pass read the states once) and the
-        # hot-path table's one-step-per-pass bytes
-        byts = metropolis_bytes(chi, s["C"], s["T"], n, lookahead=self.lookahead)
+        # the kernel's own bytes (bit-planes, two steps per pass) and the hot-path table's
+        # bytes (a 16-byte Pauli state per (chain, term), one step per pass)
+        byts = metropolis_plane_bytes(chi, s["C"], s["T"], n, tile_mf, lookahead=self.lookahead)
         byts1 = metropolis_bytes(chi, s["C"], s["T"], n)
         rows["metropolis"] = {"bound": "hbm", "achieved": byts / t / 1e9, "peak": hbm_peak, "unit": "GB/s",
                               "frac": byts / t / 1e9 / hbm_peak, "frac_formula": byts1 / t / 1e9 / hbm_peak,
@@ -1207,7 +1270,7 @@ def hidden_shift_sum8_study(local=0, chi=1 << 24, L=256, K=3):
 def hidden_shift_sum8_chain_study(local=0, chi=1 << 24, flip_steps=32, learned_steps=8, chunk=16, hidden=512,
                                   train_samples=100_000, epochs=5, exact_samples=4, L=256, K=3):
     """Chains on the 2^24-term hidden shift (16 CCZ in the 8-term form, prefactor 1/6,
-    sparsified; n = 40): 1024 single-flip chains hold 206 GB of Pauli states next to
+    sparsified; n = 40): 1024 single-flip chains hold their bit-plane states (up to 90 GB) next to
     the 17 GB tableau.  (a) every chain started at s: how many steps stay at s (P(s)
     is near 1 and every neighbour's amplitude near 0, so a move away is almost never
     accepted); (b) chains started by the term sampler of Sec. 4.2 (a term drawn by
@@ -1721,7 +1784,7 @@ def main():
                       "parallelism": f"replicas x{world}", "tuned": tuned},
            "roofline": roof, "phases": rows, "amplitude_error": err, "parity_slices": parity,
            "sparsification_certificate": cert,
-           "cpu_baseline": cpu, "cpu_baseline_python": cpu_py, "e2e": e2e, "gpu_launches": launches_per_step(r.shape["T"], r.lookahead) * args.steps,
+           "cpu_baseline": cpu, "cpu_baseline_python": cpu_py, "e2e": e2e, "gpu_launches": r.launches() * args.steps,
            "clocks": clk.summary(), "ess": ess, "side_step": side, **extra}
     print(json.dumps(out))
 

@@ -349,10 +349,10 @@ lrs_status lrs_sample_terms(lrs_ctx* ctx, int64_t count, uint64_t seed, uint64_t
                             int64_t* alpha_dev, void* stream);
 
 /* ---- Metropolis (Sec. 4.2) ------------------------------------------------------ */
-/* Start n_chains chains at x_dev[c]: computes Q_x for every (chain, term) and
- * P(x) = |<x|psi>|^2.  Needs n <= 62 (Q = i^mu X(u) Z(w) is packed in 12 bytes for
- * n <= 40, 16 bytes above).  Storage is n_chains * chi_padded * 12 (or 16) bytes,
- * owned by the context.
+/* Start n_chains chains at x_dev[c]: computes the phase and the constraints'
+ * syndromes of every (chain, term) at x and P(x) = |<x|psi>|^2.  Needs n <= 62.
+ * Storage, owned by the context: (4 + n, rounded up to even) bits per (chain, term)
+ * and (1.5 n^2 + 3 n) bits + 8 bytes per term for the terms' bit-planes.
  * Errors: LRS_ERR_ARG, LRS_ERR_STATE, LRS_ERR_UNSUPPORTED (n > 62), LRS_ERR_OOM. */
 lrs_status lrs_chains_init(lrs_ctx* ctx, int64_t n_chains, const uint64_t* x_dev, void* stream);
 
@@ -379,7 +379,7 @@ lrs_status lrs_metropolis_step(lrs_ctx* ctx, int64_t steps, uint64_t seed, int64
  *                             strings: P(x_c) = |amp_dev[c]|^2 from the summed
  *                             amplitudes (amp_dev: 2 C doubles, Re/Im; device)
  *   lrs_metropolis_propose    step `step` (global index) of lrs_metropolis_step's draws:
- *                             applies the previous step's accepted flips to the Pauli
+ *                             applies the previous step's accepted flips to the chain
  *                             states, draws j, writes the shard's sum over its terms of
  *                             b <y_c|phi> into amp_dev (2 C doubles, not squared)
  *   lrs_metropolis_accept     the FP64 accept rule of lrs_metropolis_step on the summed
@@ -560,10 +560,9 @@ lrs_status lrs_alu_probe(int32_t device, int64_t iters, double* ops_per_s);
  *                                 every term sums over y = G (s + x) restricted to the
  *                                 n - |v| constraints, on the route that its |v|
  *                                 decides, so the value changes nothing.
- *   LRS_TUNE_MC_STAGES            Metropolis: chains whose inputs a block keeps
- *                                 in flight in shared memory (1..4, 1; 12 KB each
- *                                 for one step per pass, 20 KB for two: one stage
- *                                 leaves room for the most blocks per SM)
+ *   LRS_TUNE_MC_STAGES            Metropolis (1..4, 1): accepted and returned; a block
+ *                                 copies its terms' coefficients once, so the value
+ *                                 changes nothing.
  *   LRS_TUNE_APPLY_LANES          apply_clifford for n > 48 (64-bit rows): lanes
  *                                 per term (1, 2 or 4; default 1).  The lanes of a
  *                                 term share its tableau in shared memory and split
@@ -574,13 +573,13 @@ lrs_status lrs_alu_probe(int32_t device, int64_t iters, double* ops_per_s);
  *   LRS_TUNE_NORM_FUSE_FOLDS      norm estimate (0..8, 8): accepted and returned, as
  *                                 LRS_TUNE_NORM_MAX_FOLDS; changes nothing.
  *   LRS_TUNE_MC_LOOKAHEAD         Metropolis flip chains: steps per pass over the
- *                                 chains' Pauli states (1 or 2, default 2).  With 2
+ *                                 chains' states (1 or 2, default 2).  With 2
  *                                 one pass forms <y|psi> for step t's proposal and
  *                                 for both strings step t + 1 may propose (after an
  *                                 accepted or a rejected move; proposals do not
  *                                 depend on the chain), then both decisions are taken
  *                                 in order: the same chains, bit for bit, as one step
- *                                 per pass, with half the Pauli-state reads.
+ *                                 per pass, with half the state reads.
  */
 enum {
     LRS_TUNE_AMP_BLOCKS_PER_SM = 0,

@@ -182,9 +182,10 @@ __device__ __forceinline__ int mc_row(int p, int q, int zero) {
 // and the syndromes.
 __global__ void __launch_bounds__(MC_TPB) k_mc_start(McView V, int64_t C, uint2* __restrict__ S,
                                                      const uint64_t* __restrict__ xs, uint64_t nmask, int tbx,
-                                                     int64_t tblocks) {
+                                                     int64_t cblocks) {
+    // chains fastest: the blocks that read one column range's planes run together
     const int tid = threadIdx.x;
-    const int64_t tb = blockIdx.x % tblocks, c = blockIdx.x / tblocks * (MC_TPB / tbx) + tid / tbx;
+    const int64_t tb = blockIdx.x / cblocks, c = blockIdx.x % cblocks * (MC_TPB / tbx) + tid / tbx;
     const int64_t col = tb * tbx + tid % tbx;
     if (c >= C || col >= V.cols) return;
     const uint64_t x = xs[c] & nmask;
@@ -773,9 +774,9 @@ static lrs_status mc_start(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) {
     mc_layout(ctx, &V);
     const int64_t C = ctx->n_chains;
     const int tbx = mc_columns(V.cols), nsub = MC_TPB / tbx;
-    const int64_t tblocks = (V.cols + tbx - 1) / tbx, blocks = tblocks * ((C + nsub - 1) / nsub);
+    const int64_t cblocks = (C + nsub - 1) / nsub, blocks = (V.cols + tbx - 1) / tbx * cblocks;
     if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "chain start grid too large");
-    k_mc_start<<<(unsigned)blocks, MC_TPB, 0, st>>>(V, C, (uint2*)ctx->Q, x, ctx->nmask, tbx, tblocks);
+    k_mc_start<<<(unsigned)blocks, MC_TPB, 0, st>>>(V, C, (uint2*)ctx->Q, x, ctx->nmask, tbx, cblocks);
     LRS_LAUNCH_CHECK("chain start kernel");
     double* amp = nullptr;
     lrs_status rc = launch_amplitude_start(ctx, x, C, &amp, st);

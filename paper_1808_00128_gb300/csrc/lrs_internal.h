@@ -97,9 +97,9 @@ struct lrs_ctx {
     // launch-shape tuning (lrs_set_tuning)
     int64_t tune_amp_bps = 8;       // amplitude: target blocks per SM
     int64_t tune_norm_tiles = 2048; // norm: maximum term tiles per A-block column
-    int64_t tune_mc_cg = 64;        // Metropolis: chains per block (1..64)
-    int64_t tune_mc_stages = 1;     // Metropolis: chains in flight per block (1..4)
-    int64_t tune_mc_lookahead = 2;  // Metropolis: steps per pass over the Pauli states (1, 2)
+    int64_t tune_mc_cg = 64;        // Metropolis: most chains per block (1..64)
+    int64_t tune_mc_stages = 1;     // Metropolis: no effect (kept for callers that set it; 1..4)
+    int64_t tune_mc_lookahead = 2;  // Metropolis: steps per pass over the chain states (1, 2)
     int64_t tune_norm_folds = 12;   // norm: no effect (kept for callers that set it; -1..12)
     int64_t tune_norm_fuse = 8;     // norm: no effect (kept for callers that set it; 0..8)
     int64_t tune_apply_lanes = 1;   // apply_clifford, 64-bit rows (n > 48): lanes per term (1, 2, 4)
