@@ -246,10 +246,10 @@ def launches_per_step(T, lookahead=1):
 # dram__bytes_write.sum), per unit of work, with the hash of the kernel source the
 # capture ran; `traffic` is reported only while that source is unchanged.
 TRAFFIC = {
-    # a form-per-thread k_norm on the profiling case (n = 50 QAOA, chi = 2^16, L = 64):
-    # 34,172,672 B read + 185,088 B written per launch for 2^16 x 64 (A, term) units
-    "norm_estimate": {"bytes_per_unit": (34172672 + 185088) / (65536 * 64),
-                      "source": "paper_1808_00128_gb300/csrc/k_norm.cu", "sha16": "8f42b33d2b5067dc",
+    # k_norm<52, 0> on the profiling case (n = 50 QAOA, chi = 2^16, L = 64): 35,185,664 B
+    # read + 2,357,760 B written per launch for 2^16 x 64 (A, term) units
+    "norm_estimate": {"bytes_per_unit": (35185664 + 2357760) / (65536 * 64),
+                      "source": "paper_1808_00128_gb300/csrc/k_norm.cu", "sha16": "409e8ed765041395",
                       "profile": "profiles/k_norm_n50_chi65536_L64.md"},
 }
 

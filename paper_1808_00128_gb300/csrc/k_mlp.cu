@@ -977,8 +977,8 @@ __global__ void k_logq(const float* __restrict__ logits, const uint64_t* __restr
 // either layer is evaluated once per sample: before bit i the units of degree i (H1 from the
 // bits, H2 from H1), then the logit.  A block draws all n bits of R rows with both layers'
 // activations in shared memory; H1 and H2 of later units stay zero, as their masked weights
-// are.  (A product of the whole H x H layer and a launch pair per bit took n times the work:
-// 190 us for 1024 samples at n = 20, H = 512.)
+// are.  (A product of the whole H x H layer and a launch pair per bit took n times the work: about
+// 370 us for 1024 samples at n = 20, H = 512, against 102.)
 // Bounded by latency: three barriers a bit, the weights of a bit loaded one phase ahead;
 // activations are kept as FP32 (of their BF16 roundings), so that the products are packed FP32
 // pairs without conversions.
