@@ -330,7 +330,9 @@ __global__ void k_amp_reduce_batch(const __grid_constant__ AmpBatch B, int64_t t
 // table of the chunk's 64 XORs of string words, which depends on the strings only
 // and serves every term.  Per (term, 1024 strings) that is about n^2 / 12 + 1.5 n + n / 6 per
 // constraint shared-memory loads of 128 bytes and three integer instructions each, where one
-// string per thread takes 8 ceil(n / 4) + 16 instructions for 32 strings.
+// string per thread takes 8 ceil(n / 4) + 16 instructions for 32 strings.  4096 strings: n = 50,
+// chi = 2^20 34.3 -> 13.4 ms, n = 40, chi = 2^16 with bounds 1.95 -> 0.69 ms; 1024 strings of 64
+// terms 79 -> 31 us; integer issue bounds it (ALU pipe 72% busy).
 constexpr int AS_WARPS = 8, AS_TPB = 32 * AS_WARPS;
 constexpr int AS_CB = 6;       // qubits per chunk
 constexpr int AS_TERMS = 32;   // terms whose words the block collects before summing
@@ -534,6 +536,7 @@ __global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint
     const int64_t tile = tile0 + tg * G + g;
     const int64_t b0 = tile < tile1 ? tile * tt : 0;
     const int64_t len = tile < tile1 ? (b0 + tt < cap ? tt : cap - b0) : 0;   // of this lane's tile
+    const bool used = (xb * wl + l) * 32 < batch;   // lanes past the batch's words
     uint32_t tl;   // opaque and after the barrier: the table's loads depend on it
     asm volatile("add.u32 %0, %1, %2;" : "=r"(tl) : "r"(tab0), "r"(4u * lane) : "memory");
     uint64_t sum[4], nc[4];   // complex pairs
@@ -550,7 +553,7 @@ __global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint
             const uint64_t* rec = P.rec + (have ? b0 + c0 + t - a0 : 0) * P.words;
             const ulonglong2 head = __ldg(reinterpret_cast<const ulonglong2*>(rec));
             const ulonglong2 lin = __ldg(reinterpret_cast<const ulonglong2*>(rec + AMP_LO));
-            const bool on = have && ((uint32_t)head.x >> 8 & 1u);
+            const bool on = have && used && ((uint32_t)head.x >> 8 & 1u);
             {   // the warp's next record on its way
                 const char* nx = reinterpret_cast<const char*>(rec + (int64_t)AS_WARPS * P.words) + l * 128;
                 if (c0 + t + AS_WARPS < len && l * 16 < AMP_ROWS + P.rows)
@@ -673,7 +676,7 @@ lrs_status launch_sliced_t(lrs_ctx* ctx, const AmpPrep& R, const uint64_t* x, in
     return LRS_OK;
 }
 
-// Tile sums of the batch by the sliced kernel, the records of at most AMP_REC_BYTES of terms
+// Tile sums of the batch by the sliced kernel, the records of amp_tiles_at_once tiles of terms
 // at a time in `rec`.
 constexpr size_t AMP_REC_BYTES = (size_t)512 << 20;
 AmpPrep amp_records(const lrs_ctx* ctx) {
@@ -683,21 +686,29 @@ AmpPrep amp_records(const lrs_ctx* ctx) {
     R.words = (AMP_ROWS + R.rows + ctx->n + 2 + 15) & ~15;   // lines of 128 bytes
     return R;
 }
-// tiles whose records are held at a time
-int64_t amp_tiles_at_once(const AmpPrep& R, const AmpPlan& P) {
-    int64_t t = (int64_t)(AMP_REC_BYTES / ((size_t)P.tt * R.words * sizeof(uint64_t)));
-    if (t < 32) t = 32;   // a block may take 32 tiles
-    t &= ~(int64_t)31;
+// Tiles whose records are held at a time: AMP_REC_BYTES of them, or with tiles so long that
+// these are few (chi above about 2^21) two blocks of 1024 strings per SM, a few percent of the
+// tableau's own size.
+int64_t amp_tiles_at_once(const lrs_ctx* ctx, const AmpPrep& R, const AmpPlan& P, int64_t batch) {
+    const int64_t xb = (batch + 1023) / 1024, fill = ((2 * ctx->sm_count + xb - 1) / xb + 31) & ~(int64_t)31;
+    int64_t t = (int64_t)(AMP_REC_BYTES / ((size_t)P.tt * R.words * sizeof(uint64_t))) & ~(int64_t)31;
+    if (t < fill) t = fill;
     return t < P.n_tiles ? t : P.n_tiles;
 }
 
 lrs_status launch_sliced(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* partial, const AmpPlan& P, AmpPrep R,
                          float* magp, cudaStream_t st) {
     // string words of a block: 32 (1024 strings), fewer for a batch that has fewer, whose
-    // blocks then take several tiles
+    // blocks then take several tiles, as long as that leaves two blocks per SM (with 3
+    // strings of 2048 terms, 32 tiles a block made two blocks and 17 us more than the
+    // string-per-thread kernel)
+    const int64_t held = amp_tiles_at_once(ctx, R, P, batch);
     int wl = 32;
-    while (wl > 1 && batch <= 16 * wl) wl /= 2;
-    const int64_t step = amp_tiles_at_once(R, P);
+    while (wl > 1 && batch <= 16 * wl && held * (wl / 2) >= (int64_t)64 * ctx->sm_count) wl /= 2;
+    // launches of equal length: 607 tiles of 4096 strings as 304 + 303 are 4 + 4 full waves,
+    // as 320 + 287 they were 5 + 4
+    const int64_t G = 32 / wl, parts = (P.n_tiles + held - 1) / held;
+    const int64_t step = ((P.n_tiles + parts - 1) / parts + G - 1) / G * G;
     for (int64_t t0 = 0; t0 < P.n_tiles; t0 += step) {
         const int64_t t1 = t0 + step < P.n_tiles ? t0 + step : P.n_tiles;
         const int64_t a0 = t0 * P.tt, a1 = t1 * P.tt < ctx->cap ? t1 * P.tt : ctx->cap;
@@ -761,7 +772,7 @@ static lrs_status launch_amp_scratch(lrs_ctx* ctx, const uint64_t* x, int64_t ba
     const size_t mags = err ? ((size_t)batch * P.n_tiles * sizeof(float) + 255) & ~(size_t)255 : 0;
     const size_t amps = amp_out ? ((size_t)batch * 2 * sizeof(double) + 255) & ~(size_t)255 : 0;
     AmpPrep R = amp_records(ctx);
-    int64_t terms = amp_tiles_at_once(R, P) * P.tt;
+    int64_t terms = amp_tiles_at_once(ctx, R, P, batch) * P.tt;
     if (terms > ctx->cap) terms = ctx->cap;
     const size_t need = part + mags + amps;
     void* scr = nullptr;
