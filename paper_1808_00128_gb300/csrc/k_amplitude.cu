@@ -331,7 +331,7 @@ __global__ void k_amp_reduce_batch(const __grid_constant__ AmpBatch B, int64_t t
 // and serves every term.  Per (term, 1024 strings) that is about n^2 / 12 + 1.5 n + n / 6 per
 // constraint shared-memory loads of 128 bytes and three integer instructions each, where one
 // string per thread takes 8 ceil(n / 4) + 16 instructions for 32 strings.  4096 strings: n = 50,
-// chi = 2^20 34.3 -> 13.4 ms, n = 40, chi = 2^16 with bounds 1.95 -> 0.69 ms; 1024 strings of 64
+// chi = 2^20 34.3 -> 12.0 ms, n = 40, chi = 2^16 with bounds 1.95 -> 0.69 ms; 1024 strings of 64
 // terms 79 -> 31 us; integer issue bounds it (ALU pipe 72% busy).
 constexpr int AS_WARPS = 8, AS_TPB = 32 * AS_WARPS;
 constexpr int AS_CB = 6;       // qubits per chunk
@@ -699,12 +699,13 @@ int64_t amp_tiles_at_once(const lrs_ctx* ctx, const AmpPrep& R, const AmpPlan& P
 lrs_status launch_sliced(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* partial, const AmpPlan& P, AmpPrep R,
                          float* magp, cudaStream_t st) {
     // string words of a block: 32 (1024 strings), fewer for a batch that has fewer, whose
-    // blocks then take several tiles, as long as that leaves two blocks per SM (with 3
-    // strings of 2048 terms, 32 tiles a block made two blocks and 17 us more than the
-    // string-per-thread kernel)
+    // blocks then take several tiles, as long as that leaves a block per SM (gates and 100
+    // amplitudes of 300001 terms: 5.57 ms, with two blocks per SM 5.79 ms; with 3 strings of
+    // 2048 terms, 32 tiles a block made two blocks and 17 us more than the string-per-thread
+    // kernel)
     const int64_t held = amp_tiles_at_once(ctx, R, P, batch);
     int wl = 32;
-    while (wl > 1 && batch <= 16 * wl && held * (wl / 2) >= (int64_t)64 * ctx->sm_count) wl /= 2;
+    while (wl > 1 && batch <= 16 * wl && held * (wl / 2) >= (int64_t)32 * ctx->sm_count) wl /= 2;
     // launches of equal length: 607 tiles of 4096 strings as 304 + 303 are 4 + 4 full waves,
     // as 320 + 287 they were 5 + 4
     const int64_t G = 32 / wl, parts = (P.n_tiles + held - 1) / held;
