@@ -526,6 +526,9 @@ lrs_status lrs_metropolis_learned(lrs_ctx* ctx, lrs_mlp* mlp, int64_t steps, uin
  *                                      lrs_mlp_set_gemm then returns LRS_ERR_TIMEOUT
  * A later call of the same kind runs normally.                                       */
 lrs_status lrs_debug_inject_wait_timeout(lrs_ctx* ctx);
+/* From now on an allocation of ctx's scratch or chain buffers of more than `bytes`
+ * fails with the status of a failed cudaMalloc, without being tried (0: no limit). */
+lrs_status lrs_debug_limit_alloc(lrs_ctx* ctx, int64_t bytes);
 lrs_status lrs_mlp_debug_inject_wait_timeout(lrs_mlp* mlp);
 
 /* ---- export (checkpoint / bit-exact parity) ----------------------------------- */

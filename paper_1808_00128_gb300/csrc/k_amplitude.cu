@@ -779,10 +779,7 @@ static lrs_status launch_amp_scratch(lrs_ctx* ctx, const uint64_t* x, int64_t ba
     void* scr = nullptr;
     lrs_status rc = lrs_scratch(ctx, need + (size_t)terms * R.words * sizeof(uint64_t), &scr);
     const bool sliced = rc == LRS_OK;
-    if (rc == LRS_ERR_OOM) {
-        cudaGetLastError();   // the failed allocation's error is not the next launch's
-        rc = lrs_scratch(ctx, need, &scr);
-    }
+    if (rc == LRS_ERR_OOM) rc = lrs_scratch(ctx, need, &scr);
     if (rc != LRS_OK) return rc;
     float2* partial = (float2*)scr;
     float* magp = err ? (float*)((char*)scr + part) : nullptr;

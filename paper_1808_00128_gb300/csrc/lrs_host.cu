@@ -21,13 +21,14 @@ lrs_status lrs_fail(lrs_status st, const char* fmt, ...) {
 }
 
 lrs_status lrs_cuda_check(cudaError_t e, const char* what) {
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();   // reported here, not by the next launch's check
     return lrs_fail(e == cudaErrorMemoryAllocation ? LRS_ERR_OOM : LRS_ERR_CUDA, "%s: %s", what,
                     cudaGetErrorString(e));
 }
 
 extern "C" const char* lrs_last_error(void) { return g_err; }
 
-lrs_status lrs_ensure(void** ptr, size_t* have, size_t bytes) {
+lrs_status lrs_ensure(void** ptr, size_t* have, size_t bytes, size_t limit) {
     if (*have >= bytes && *ptr) return LRS_OK;
     if (*ptr) {
         cudaFree(*ptr);
@@ -35,7 +36,7 @@ lrs_status lrs_ensure(void** ptr, size_t* have, size_t bytes) {
         *have = 0;
     }
     if (bytes == 0) return LRS_OK;
-    cudaError_t e = cudaMalloc(ptr, bytes);
+    cudaError_t e = limit && bytes > limit ? cudaErrorMemoryAllocation : cudaMalloc(ptr, bytes);
     if (e != cudaSuccess) {
         *ptr = nullptr;
         return lrs_cuda_check(e, "cudaMalloc");
@@ -45,7 +46,7 @@ lrs_status lrs_ensure(void** ptr, size_t* have, size_t bytes) {
 }
 
 lrs_status lrs_scratch(lrs_ctx* ctx, size_t bytes, void** out) {
-    lrs_status rc = lrs_ensure(&ctx->scratch, &ctx->scratch_bytes, bytes);
+    lrs_status rc = lrs_ensure(&ctx->scratch, &ctx->scratch_bytes, bytes, ctx->alloc_limit);
     *out = ctx->scratch;
     return rc;
 }
@@ -878,9 +879,10 @@ extern "C" lrs_status lrs_chains_init(lrs_ctx* c, int64_t n_chains, const uint64
     if (n_chains < 1 || !x) return lrs_fail(LRS_ERR_ARG, "bad chains");
     if (n_chains > 65535) return lrs_fail(LRS_ERR_ARG, "at most 65535 chains");
     LRS_CUDA(cudaSetDevice(c->device));
-    lrs_status rc = lrs_ensure((void**)&c->Q, &c->Q_bytes, mc_state_bytes(c, n_chains));
+    c->n_chains = 0;   // until every buffer is there and set: no steps on the chains of a failed call
+    lrs_status rc = lrs_ensure((void**)&c->Q, &c->Q_bytes, mc_state_bytes(c, n_chains), c->alloc_limit);
     if (rc != LRS_OK) return rc;
-    rc = lrs_ensure(&c->mc_planes, &c->mc_planes_bytes, mc_planes_bytes(c));
+    rc = lrs_ensure(&c->mc_planes, &c->mc_planes_bytes, mc_planes_bytes(c), c->alloc_limit);
     if (rc != LRS_OK) return rc;
     if (n_chains > c->chains_cap) {
         cudaFree(c->cx); cudaFree(c->cp); cudaFree(c->pend);
@@ -894,7 +896,9 @@ extern "C" lrs_status lrs_chains_init(lrs_ctx* c, int64_t n_chains, const uint64
     c->n_chains = n_chains;
     c->q_stale = false;
     c->split_step = -1;
-    return launch_chains_init(c, x, as_stream(stream));
+    rc = launch_chains_init(c, x, as_stream(stream));
+    if (rc != LRS_OK) c->n_chains = 0;
+    return rc;
 }
 
 extern "C" lrs_status lrs_metropolis_step(lrs_ctx* c, int64_t steps, uint64_t seed, int64_t step0,
@@ -959,6 +963,13 @@ extern "C" lrs_status lrs_debug_inject_wait_timeout(lrs_ctx* c) {
     lrs_status rc = mc_flags(c);
     if (rc != LRS_OK) return rc;
     *(volatile int*)&c->mc_err_h[1] = 1;
+    return LRS_OK;
+}
+
+extern "C" lrs_status lrs_debug_limit_alloc(lrs_ctx* c, int64_t bytes) {
+    if (!c) return lrs_fail(LRS_ERR_ARG, "ctx is NULL");
+    if (bytes < 0) return lrs_fail(LRS_ERR_ARG, "bytes < 0");
+    c->alloc_limit = (size_t)bytes;
     return LRS_OK;
 }
 

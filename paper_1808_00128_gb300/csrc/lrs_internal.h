@@ -94,6 +94,7 @@ struct lrs_ctx {
     // scratch for partial sums
     void* scratch = nullptr;
     size_t scratch_bytes = 0;
+    size_t alloc_limit = 0;         // lrs_debug_limit_alloc: larger buffers fail to allocate (0: none)
     // launch-shape tuning (lrs_set_tuning)
     int64_t tune_amp_bps = 8;       // amplitude: target blocks per SM
     int64_t tune_norm_tiles = 2048; // norm: maximum term tiles per A-block column
@@ -162,8 +163,9 @@ lrs_status lrs_cuda_check(cudaError_t e, const char* what);
         if (e_ != cudaSuccess) return lrs_cuda_check(e_, what);     \
     } while (0)
 
-// Grow a device buffer to at least `bytes` (contents not kept).
-lrs_status lrs_ensure(void** ptr, size_t* have, size_t bytes);
+// Grow a device buffer to at least `bytes` (contents not kept).  limit (0: none): a larger
+// allocation fails as cudaMalloc would, without being tried (lrs_debug_limit_alloc).
+lrs_status lrs_ensure(void** ptr, size_t* have, size_t bytes, size_t limit = 0);
 lrs_status lrs_scratch(lrs_ctx* ctx, size_t bytes, void** out);
 // True while `st` is being captured into a CUDA graph: launches then skip the one-time
 // function-attribute calls (made by an earlier uncaptured call) and nested graphs.

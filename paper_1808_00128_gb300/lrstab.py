@@ -44,7 +44,7 @@ EXPORTED = ["lrs_lower_circuit", "lrs_create", "lrs_destroy", "lrs_last_error", 
             "lrs_apply_circuit_shared", "lrs_decomposition_stats", "lrs_sparsification_certificate",
             "lrs_debug_inject_wait_timeout", "lrs_mlp_debug_inject_wait_timeout", "lrs_chains_set_amplitude",
             "lrs_metropolis_propose", "lrs_metropolis_accept", "lrs_norm_overlaps",
-            "lrs_norm_eta_from_overlaps", "lrs_amplitude_batch"]
+            "lrs_norm_eta_from_overlaps", "lrs_amplitude_batch", "lrs_debug_limit_alloc"]
 
 
 class LrsError(RuntimeError):
@@ -106,6 +106,7 @@ def lib():
         "lrs_decomposition_stats": [vp, i64, vp, vp, vp],
         "lrs_sparsification_certificate": [vp, i64, i32, u64, vp, vp],
         "lrs_debug_inject_wait_timeout": [vp],
+        "lrs_debug_limit_alloc": [vp, i64],
         "lrs_mlp_debug_inject_wait_timeout": [vp],
         "lrs_chains_set_amplitude": [vp, vp, vp],
         "lrs_metropolis_propose": [vp, u64, i64, vp, vp],
@@ -435,6 +436,10 @@ class Simulator:
     def debug_inject_wait_timeout(self):
         """lrs_debug_inject_wait_timeout (failure-path tests)."""
         _check(lib().lrs_debug_inject_wait_timeout(self._h))
+
+    def debug_limit_alloc(self, size: int):
+        """lrs_debug_limit_alloc (failure-path tests): larger buffers fail to allocate."""
+        _check(lib().lrs_debug_limit_alloc(self._h, size))
 
     def export_terms(self, first: int = 0, count: int | None = None) -> dict:
         count = self.chi - first if count is None else count
