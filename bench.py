@@ -213,16 +213,20 @@ def metropolis_plane_bytes(chi, C, T, n, mf, accept=0.5, lookahead=1):
     return passes * (C * chi / 64 * 8 * words + chi * (planes / 8 + 8))
 
 
-def record_launches(n, chi, B, per_block, sms=152, blocks_per_sm=8):
-    """Launches of the amplitude records and sums (two per 512 MB of records)."""
+def record_launches(n, chi, B, per_block, sms, blocks_per_sm=8):
+    """Launches of the amplitude records and sums: two per part of every term tile whose
+    records fit 512 MB (amp_plan and amp_range of k_amplitude.cu)."""
     cap = (chi + 255) // 256 * 256
     xblocks = (B + per_block - 1) // per_block
     nt = max(1, min((sms * blocks_per_sm + xblocks - 1) // xblocks, (cap + 31) // 32))
     tt = ((cap + nt - 1) // nt + 7) // 8 * 8
     tiles = (cap + tt - 1) // tt
     words = (4 + (n + 5) // 6 * 6 + n + 2 + 15) // 16 * 16
-    step = max(32, (512 << 20) // (tt * words * 8)) // 32 * 32
-    return 2 * ((tiles + step - 1) // step)
+    held = (512 << 20) // (words * 8)
+    if held >= cap:
+        return 2
+    most = held // tiles // 32 * 32
+    return 2 * ((tt + most - 1) // most)
 
 
 def units_per_step(chi, B, C, T):
@@ -596,8 +600,12 @@ class StepRunner:
     def launches(self):
         """Library kernels one step launches."""
         s = self.shape
-        return (launches_per_step(s["T"], self.lookahead) + record_launches(self.n, self.chi, s["B"], 1024) - 1
-                + 2 + record_launches(self.n, self.chi, s["C"], 512) - 1)
+        if getattr(self, "_bps", None) is None:
+            import torch
+            self._bps = (torch.cuda.get_device_properties(self.dev).multi_processor_count,
+                         self.sim.get_tuning("amp_blocks_per_sm"))
+        return (launches_per_step(s["T"], self.lookahead) + record_launches(self.n, self.chi, s["B"], 1024, *self._bps) - 1
+                + 2 + record_launches(self.n, self.chi, s["C"], 512, *self._bps) - 1)
 
     def rooflines(self, phase_ms, alu_peak, hbm_peak):
         """Per phase: achieved and fraction of the roofline on the kernel's own op count

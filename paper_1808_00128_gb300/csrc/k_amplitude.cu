@@ -339,19 +339,24 @@ constexpr int AS_TERMS = 32;   // terms whose words the block collects before su
 enum { AMP_INFO = 0, AMP_VAL, AMP_LO, AMP_HI, AMP_ROWS };   // record: header, rows L_0.., constraints
 
 struct AmpPrep {
-    uint64_t* rec;   // [terms][words]
-    int words, rows; // rows = chunks * AS_CB
+    uint64_t* rec;   // [slots][words]
+    int words, rows;   // rows = chunks * AS_CB
+    // the launch's terms: r0 .. r0 + rl - 1 of every tile of tt terms; term r0 + j of tile t in
+    // slot t rl + j
+    int64_t tt, r0;
+    int rl;
 };
 
-// Records of terms [a0, a0 + count): a warp per term, lane c holding rows c and c + 32.
-__global__ void __launch_bounds__(256) k_amp_prep(TermsView T, int64_t a0, int64_t count, AmpPrep P) {
+// Records of a launch's terms, eight terms of tile blockIdx.y a block (rl is a multiple of 8): a
+// warp per term, lane c holding rows c and c + 32.
+__global__ void __launch_bounds__(256) k_amp_prep(TermsView T, AmpPrep P) {
     __shared__ uint64_t sF[8][64];
     const int n = T.n, lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), a = a0 + i;
-    if (i >= count) return;
+    const int64_t j = blockIdx.x * 8 + (threadIdx.x >> 5), r = P.r0 + j, a = (int64_t)blockIdx.y * P.tt + r;
+    if (r >= P.tt || a >= T.cap) return;
     const uint64_t v = T.v[a], s = T.s[a], glo = T.glo[a], ghi = T.ghi[a];
     const uint32_t om = T.omega[a];
-    uint64_t* rec = P.rec + i * P.words;
+    uint64_t* rec = P.rec + ((int64_t)blockIdx.y * P.rl + j) * P.words;
     const bool live = ((om >> 3) & 1u) == 0u;
     const uint64_t out = ~v & T.nmask;
     const int mf = __popcll(out);
@@ -491,13 +496,14 @@ __device__ __forceinline__ void kahan_add2(uint64_t& s, uint64_t& nc, float x, f
 // word l for tile g.  The warps first evaluate AS_TERMS terms of every tile, one term each at
 // a time, leaving three words per lane and term (live, phase bits); then thread (warp, lane)
 // adds up the four strings 4 warp .. 4 warp + 3 of its lane's word, in term order, so every
-// string's Kahan sum over a tile is the one a single thread would form.
+// string's Kahan sum over a tile is the one a single thread would form; a sum that a later
+// launch continues (more) is left as it stands, its compensation in `comp`.
 // The table takes 8 KB per chunk (72 KB at n = 50): two blocks an SM.
 template <int NC, bool ERR>
 __global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint64_t nmask, const uint64_t* __restrict__ xs,
-                                                          int64_t batch, int64_t tt, int64_t cap, int64_t a0, int64_t tile0,
-                                                          int64_t tile1, int64_t n_tiles, int wl, int64_t tgroups,
-                                                          float2* __restrict__ partial, float* __restrict__ magp) {
+                                                          int64_t batch, int64_t cap, int64_t n_tiles, int wl,
+                                                          int64_t tgroups, bool more, float2* __restrict__ partial,
+                                                          float2* __restrict__ comp, float* __restrict__ magp) {
     // shared memory: table (on an 8 KB boundary), then the collected words and values, whose
     // place holds the string words while the table is built
     extern __shared__ __align__(16) unsigned char dyn[];
@@ -533,9 +539,11 @@ __global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint
         }
     }
     __syncthreads();
-    const int64_t tile = tile0 + tg * G + g;
-    const int64_t b0 = tile < tile1 ? tile * tt : 0;
-    const int64_t len = tile < tile1 ? (b0 + tt < cap ? tt : cap - b0) : 0;   // of this lane's tile
+    const int64_t tile = tg * G + g;
+    // this launch's terms of this lane's tile, and the slot of the first
+    const int64_t end = tile < n_tiles ? (tile * P.tt + P.tt < cap ? P.tt : cap - tile * P.tt) - P.r0 : 0;
+    const int len = end < P.rl ? (int)end : P.rl;   // 0 or less: none
+    const int64_t slot0 = tile * P.rl;
     const bool used = (xb * wl + l) * 32 < batch;   // lanes past the batch's words
     uint32_t tl;   // opaque and after the barrier: the table's loads depend on it
     asm volatile("add.u32 %0, %1, %2;" : "=r"(tl) : "r"(tab0), "r"(4u * lane) : "memory");
@@ -545,12 +553,18 @@ __global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint
     for (int k = 0; k < 4; ++k) {
         sum[k] = nc[k] = 0;
         mag[k] = 0.f;
+        const int64_t i = (xb * wl + l) * 32 + 4 * warp + k;
+        if (P.r0 > 0 && tile < n_tiles && i < batch) {   // as the launch before left them
+            sum[k] = reinterpret_cast<const uint64_t*>(partial)[i * n_tiles + tile];
+            nc[k] = reinterpret_cast<const uint64_t*>(comp)[i * n_tiles + tile];
+            if (ERR) mag[k] = magp[i * n_tiles + tile];
+        }
     }
-    for (int64_t c0 = 0; c0 < tt; c0 += AS_TERMS) {
+    for (int c0 = 0; c0 < P.rl; c0 += AS_TERMS) {
 #pragma unroll 1
-        for (int t = warp; t < AS_TERMS && c0 + t < tt; t += AS_WARPS) {
+        for (int t = warp; t < AS_TERMS && c0 + t < P.rl; t += AS_WARPS) {
             const bool have = c0 + t < len;
-            const uint64_t* rec = P.rec + (have ? b0 + c0 + t - a0 : 0) * P.words;
+            const uint64_t* rec = P.rec + (have ? slot0 + c0 + t : 0) * P.words;
             const ulonglong2 head = __ldg(reinterpret_cast<const ulonglong2*>(rec));
             const ulonglong2 lin = __ldg(reinterpret_cast<const ulonglong2*>(rec + AMP_LO));
             const bool on = have && used && ((uint32_t)head.x >> 8 & 1u);
@@ -592,7 +606,7 @@ __global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint
         }
         __syncthreads();
 #pragma unroll 1
-        for (int t = 0; t < AS_TERMS && c0 + t < tt; ++t) {
+        for (int t = 0; t < AS_TERMS && c0 + t < P.rl; ++t) {
             const uint32_t live = sw[t][0][lane] >> (4 * warp) & 15u;
             if (!__any_sync(0xffffffffu, live != 0u)) continue;
             const uint32_t q0 = sw[t][1][lane] >> (4 * warp), q1 = sw[t][2][lane] >> (4 * warp);
@@ -608,14 +622,19 @@ __global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint
         }
         __syncthreads();
     }
-    if (tile < tile1) {
+    if (tile < n_tiles) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int64_t i = (xb * wl + l) * 32 + 4 * warp + k;
             if (i < batch) {
-                partial[i * n_tiles + tile] =
-                    make_float2(__uint_as_float((uint32_t)sum[k]) + __uint_as_float((uint32_t)nc[k]),
-                                __uint_as_float((uint32_t)(sum[k] >> 32)) + __uint_as_float((uint32_t)(nc[k] >> 32)));
+                if (more) {
+                    reinterpret_cast<uint64_t*>(partial)[i * n_tiles + tile] = sum[k];
+                    reinterpret_cast<uint64_t*>(comp)[i * n_tiles + tile] = nc[k];
+                } else {
+                    partial[i * n_tiles + tile] =
+                        make_float2(__uint_as_float((uint32_t)sum[k]) + __uint_as_float((uint32_t)nc[k]),
+                                    __uint_as_float((uint32_t)(sum[k] >> 32)) + __uint_as_float((uint32_t)(nc[k] >> 32)));
+                }
                 if (ERR) magp[i * n_tiles + tile] = mag[k];
             }
         }
@@ -659,75 +678,87 @@ lrs_status launch_amp_t(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* 
 }
 
 template <int NC>
-lrs_status launch_sliced_t(lrs_ctx* ctx, const AmpPrep& R, const uint64_t* x, int64_t batch, const AmpPlan& P, int64_t a0,
-                           int64_t tile0, int64_t tile1, int wl, float2* partial, float* magp, cudaStream_t st) {
+lrs_status launch_sliced_t(lrs_ctx* ctx, const AmpPrep& R, const uint64_t* x, int64_t batch, const AmpPlan& P, int wl,
+                           float2* partial, float2* comp, float* magp, cudaStream_t st) {
     // up to 8 KB to the table's boundary, the table, the collected words and values
     const size_t smem = 8192 + (size_t)NC * 8192 +
                         (size_t)AS_TERMS * 32 * (3 * sizeof(uint32_t) + sizeof(float2) + (magp ? sizeof(float) : 0));
     const auto kernel = magp ? k_amp_sliced<NC, true> : k_amp_sliced<NC, false>;
     if (!lrs_capturing(st))
         LRS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int64_t G = 32 / wl, tgroups = (tile1 - tile0 + G - 1) / G;
+    const int64_t G = 32 / wl, tgroups = (P.n_tiles + G - 1) / G;
     const int64_t blocks = tgroups * ((batch + 32 * wl - 1) / (32 * wl));
     if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "amplitude grid too large");
-    kernel<<<(unsigned)blocks, AS_TPB, smem, st>>>(R, ctx->n, ctx->nmask, x, batch, P.tt, ctx->cap, a0, tile0, tile1,
-                                                   P.n_tiles, wl, tgroups, partial, magp);
+    kernel<<<(unsigned)blocks, AS_TPB, smem, st>>>(R, ctx->n, ctx->nmask, x, batch, ctx->cap, P.n_tiles, wl, tgroups,
+                                                   R.r0 + R.rl < P.tt, partial, comp, magp);
     LRS_LAUNCH_CHECK("amplitude kernel");
     return LRS_OK;
 }
 
-// Tile sums of the batch by the sliced kernel, the records of amp_tiles_at_once tiles of terms
-// at a time in `rec`.
+// Scratch of a call.  What it needs must not shrink as the batch grows, or a call of fewer strings
+// would reallocate the scratch that a captured call still addresses: so the partial sums are
+// counted by a bound that grows with the batch, and the records are as many for every batch.
+//
+// Partial sums of at most `batch` strings: n_tiles <= ceil(target / xblocks), and never more than
+// target or cap / 32 (the sums themselves: 1024 x 1216 at 1024 strings, 4097 x 244 at 4097).
+size_t amp_partials(const lrs_ctx* ctx, int64_t batch) {
+    const int64_t target = (int64_t)ctx->sm_count * ctx->tune_amp_bps, maxt = (ctx->cap + 31) / 32;
+    const int64_t a = batch * (target < maxt ? target : maxt), b = AMP_XB * (target + (batch + AMP_XB - 1) / AMP_XB);
+    return (size_t)(a < b ? a : b);
+}
+// Records: of all terms, or AMP_REC_BYTES of them; a call then takes several launches, each over
+// some terms of every tile.
 constexpr size_t AMP_REC_BYTES = (size_t)512 << 20;
-AmpPrep amp_records(const lrs_ctx* ctx) {
+AmpPrep amp_records(const lrs_ctx* ctx, int64_t* count) {
     AmpPrep R;
-    R.rec = nullptr;
+    memset(&R, 0, sizeof(R));
     R.rows = (ctx->n + AS_CB - 1) / AS_CB * AS_CB;
     R.words = (AMP_ROWS + R.rows + ctx->n + 2 + 15) & ~15;   // lines of 128 bytes
+    const int64_t most = (int64_t)(AMP_REC_BYTES / (R.words * sizeof(uint64_t)));
+    *count = ctx->cap < most ? ctx->cap : most;
     return R;
 }
-// Tiles whose records are held at a time: AMP_REC_BYTES of them, or with tiles so long that
-// these are few (chi above about 2^21) two blocks of 1024 strings per SM, a few percent of the
-// tableau's own size.
-int64_t amp_tiles_at_once(const lrs_ctx* ctx, const AmpPrep& R, const AmpPlan& P, int64_t batch) {
-    const int64_t xb = (batch + 1023) / 1024, fill = ((2 * ctx->sm_count + xb - 1) / xb + 31) & ~(int64_t)31;
-    int64_t t = (int64_t)(AMP_REC_BYTES / ((size_t)P.tt * R.words * sizeof(uint64_t))) & ~(int64_t)31;
-    if (t < fill) t = fill;
-    return t < P.n_tiles ? t : P.n_tiles;
+// Terms of a tile per launch with `count` slots: all, or equal parts that are whole rounds of
+// AS_TERMS (0: not even one round).
+int amp_range(const AmpPlan& P, int64_t cap, int64_t count) {
+    if (count >= cap) return (int)P.tt;
+    const int64_t most = count / P.n_tiles / AS_TERMS * AS_TERMS;
+    if (most == 0) return 0;
+    const int64_t parts = (P.tt + most - 1) / most;
+    return (int)(((P.tt + parts - 1) / parts + AS_TERMS - 1) / AS_TERMS * AS_TERMS);
 }
 
-lrs_status launch_sliced(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* partial, const AmpPlan& P, AmpPrep R,
-                         float* magp, cudaStream_t st) {
+// Tile sums of the batch by the sliced kernel, R.rl terms of every tile at a time.  (Some whole
+// tiles at a time either left too few blocks for the GPU or took records for a quarter of the
+// terms, 3.2 GB at n = 40, chi = 2^24, and reached fewer string words a block: 41 strings
+// there 46.4 -> 25.2 ms, 1024 strings 54.7 -> 55.0; 4096 strings at n = 50, chi = 2^20 12.0 ms
+// either way.)
+lrs_status launch_sliced(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* partial, float2* comp, const AmpPlan& P,
+                         AmpPrep R, float* magp, cudaStream_t st) {
     // string words of a block: 32 (1024 strings), fewer for a batch that has fewer, whose
     // blocks then take several tiles, as long as that leaves a block per SM (gates and 100
     // amplitudes of 300001 terms: 5.57 ms, with two blocks per SM 5.79 ms; with 3 strings of
     // 2048 terms, 32 tiles a block made two blocks and 17 us more than the string-per-thread
     // kernel)
-    const int64_t held = amp_tiles_at_once(ctx, R, P, batch);
     int wl = 32;
-    while (wl > 1 && batch <= 16 * wl && held * (wl / 2) >= (int64_t)32 * ctx->sm_count) wl /= 2;
-    // launches of equal length: 607 tiles of 4096 strings as 304 + 303 are 4 + 4 full waves,
-    // as 320 + 287 they were 5 + 4
-    const int64_t G = 32 / wl, parts = (P.n_tiles + held - 1) / held;
-    const int64_t step = ((P.n_tiles + parts - 1) / parts + G - 1) / G * G;
-    for (int64_t t0 = 0; t0 < P.n_tiles; t0 += step) {
-        const int64_t t1 = t0 + step < P.n_tiles ? t0 + step : P.n_tiles;
-        const int64_t a0 = t0 * P.tt, a1 = t1 * P.tt < ctx->cap ? t1 * P.tt : ctx->cap;
-        k_amp_prep<<<(unsigned)((a1 - a0 + 7) / 8), 256, 0, st>>>(ctx->view(), a0, a1 - a0, R);
+    while (wl > 1 && batch <= 16 * wl && P.n_tiles * (wl / 2) >= (int64_t)32 * ctx->sm_count) wl /= 2;
+    R.tt = P.tt;
+    for (R.r0 = 0; R.r0 < P.tt; R.r0 += R.rl) {
+        k_amp_prep<<<dim3((unsigned)(R.rl / 8), (unsigned)P.n_tiles), 256, 0, st>>>(ctx->view(), R);
         LRS_LAUNCH_CHECK("amplitude prep kernel");
         lrs_status rc;
         switch (R.rows / AS_CB) {
-            case 1: rc = launch_sliced_t<1>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 2: rc = launch_sliced_t<2>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 3: rc = launch_sliced_t<3>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 4: rc = launch_sliced_t<4>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 5: rc = launch_sliced_t<5>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 6: rc = launch_sliced_t<6>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 7: rc = launch_sliced_t<7>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 8: rc = launch_sliced_t<8>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 9: rc = launch_sliced_t<9>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            case 10: rc = launch_sliced_t<10>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
-            default: rc = launch_sliced_t<11>(ctx, R, x, batch, P, a0, t0, t1, wl, partial, magp, st); break;
+            case 1: rc = launch_sliced_t<1>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 2: rc = launch_sliced_t<2>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 3: rc = launch_sliced_t<3>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 4: rc = launch_sliced_t<4>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 5: rc = launch_sliced_t<5>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 6: rc = launch_sliced_t<6>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 7: rc = launch_sliced_t<7>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 8: rc = launch_sliced_t<8>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 9: rc = launch_sliced_t<9>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            case 10: rc = launch_sliced_t<10>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
+            default: rc = launch_sliced_t<11>(ctx, R, x, batch, P, wl, partial, comp, magp, st); break;
         }
         if (rc != LRS_OK) return rc;
     }
@@ -765,28 +796,40 @@ lrs_status launch_amp_kernels(lrs_ctx* ctx, const uint64_t* x, int64_t batch, do
 
 }  // namespace
 
-// The sliced kernels and the reduction, with scratch for partial sums, bounds (err), amplitudes
-// (*amp_out) and records; the string-per-thread kernel where the records do not fit.
+// The sliced kernels and the reduction, with scratch for partial sums and their compensations,
+// bounds (err), amplitudes (*amp_out) and records; the string-per-thread kernel where that does
+// not fit, with scratch for no more than its sums.
 static lrs_status launch_amp_scratch(lrs_ctx* ctx, const uint64_t* x, int64_t batch, const AmpPlan& P, double* out,
                                      double** amp_out, float* err, cudaStream_t st) {
-    const size_t part = ((size_t)batch * P.n_tiles * sizeof(float2) + 255) & ~(size_t)255;
-    const size_t mags = err ? ((size_t)batch * P.n_tiles * sizeof(float) + 255) & ~(size_t)255 : 0;
-    const size_t amps = amp_out ? ((size_t)batch * 2 * sizeof(double) + 255) & ~(size_t)255 : 0;
-    AmpPrep R = amp_records(ctx);
-    int64_t terms = amp_tiles_at_once(ctx, R, P, batch) * P.tt;
-    if (terms > ctx->cap) terms = ctx->cap;
-    const size_t need = part + mags + amps;
+    auto round = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
+    const size_t amps = round((size_t)batch * 2 * sizeof(double));
+    // bounds and amplitudes have their place in every call, as the sums do
+    size_t sums = amp_partials(ctx, batch), need = 2 * round(sums * sizeof(float2)) + round(sums * sizeof(float)) + amps;
+    int64_t records;
+    AmpPrep R = amp_records(ctx, &records);
     void* scr = nullptr;
-    lrs_status rc = lrs_scratch(ctx, need + (size_t)terms * R.words * sizeof(uint64_t), &scr);
+    lrs_status rc = lrs_scratch(ctx, need + (size_t)records * R.words * sizeof(uint64_t), &scr);
     const bool sliced = rc == LRS_OK;
-    if (rc == LRS_ERR_OOM) rc = lrs_scratch(ctx, need, &scr);
+    if (rc == LRS_ERR_OOM) {
+        sums = (size_t)batch * P.n_tiles;
+        need = round(sums * sizeof(float2)) + (err ? round(sums * sizeof(float)) : 0) + (amp_out ? amps : 0);
+        rc = lrs_scratch(ctx, need, &scr);
+    }
     if (rc != LRS_OK) return rc;
-    float2* partial = (float2*)scr;
-    float* magp = err ? (float*)((char*)scr + part) : nullptr;
-    if (amp_out) out = *amp_out = (double*)((char*)scr + part + mags);
+    char* at = (char*)scr;
+    auto take = [&](size_t bytes) {
+        char* q = at;
+        at += round(bytes);
+        return q;
+    };
+    float2* partial = (float2*)take(sums * sizeof(float2));
+    float* magp = err ? (float*)take(sums * sizeof(float)) : nullptr;
+    if (amp_out) out = *amp_out = (double*)take(amps);
     if (!sliced) return launch_amp_kernels(ctx, x, batch, out, partial, P, st, magp, err);
+    float2* comp = (float2*)take(sums * sizeof(float2));
     R.rec = (uint64_t*)((char*)scr + need);
-    if ((rc = launch_sliced(ctx, x, batch, partial, P, R, magp, st)) != LRS_OK) return rc;
+    R.rl = amp_range(P, ctx->cap, records);
+    if ((rc = launch_sliced(ctx, x, batch, partial, comp, P, R, magp, st)) != LRS_OK) return rc;
     k_amp_reduce<<<(unsigned)batch, 256, 0, st>>>(partial, magp, P.n_tiles, batch, P.tt, out, err);
     LRS_LAUNCH_CHECK("amplitude reduce kernel");
     return LRS_OK;
@@ -849,7 +892,7 @@ lrs_status launch_amplitude_batch(lrs_ctx* const* ctxs, const uint64_t* const* x
             const AmpPlan P = amp_plan(c, batch[i], AMP_XB);
             if (P.xblocks > 65535) return lrs_fail(LRS_ERR_UNSUPPORTED, "amplitude batch too large");
             void* scr = nullptr;
-            lrs_status rc = lrs_scratch(c, (size_t)batch[i] * P.n_tiles * sizeof(float2), &scr);
+            lrs_status rc = lrs_scratch(c, amp_partials(c, batch[i]) * sizeof(float2), &scr);
             if (rc != LRS_OK) return rc;
             B.first[k] = blocks;
             B.T[k] = c->view();
