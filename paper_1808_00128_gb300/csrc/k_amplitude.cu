@@ -723,7 +723,7 @@ AmpPrep amp_records(const lrs_ctx* ctx, int64_t* count) {
 int amp_range(const AmpPlan& P, int64_t cap, int64_t count) {
     if (count >= cap) return (int)P.tt;
     const int64_t most = count / P.n_tiles / AS_TERMS * AS_TERMS;
-    if (most == 0) return 0;
+    if (most <= 0) return 0;
     const int64_t parts = (P.tt + most - 1) / most;
     return (int)(((P.tt + parts - 1) / parts + AS_TERMS - 1) / AS_TERMS * AS_TERMS);
 }
@@ -731,7 +731,7 @@ int amp_range(const AmpPlan& P, int64_t cap, int64_t count) {
 // Tile sums of the batch by the sliced kernel, R.rl terms of every tile at a time.  (Some whole
 // tiles at a time either left too few blocks for the GPU or took records for a quarter of the
 // terms, 3.2 GB at n = 40, chi = 2^24, and reached fewer string words a block: 41 strings
-// there 46.4 -> 25.2 ms, 1024 strings 54.7 -> 55.0; 4096 strings at n = 50, chi = 2^20 12.0 ms
+// there 46.4 -> 24.5 ms, 1024 strings 54.7 -> 54.9; 4096 strings at n = 50, chi = 2^20 12.0 ms
 // either way.)
 lrs_status launch_sliced(lrs_ctx* ctx, const uint64_t* x, int64_t batch, float2* partial, float2* comp, const AmpPlan& P,
                          AmpPrep R, float* magp, cudaStream_t st) {
@@ -796,27 +796,52 @@ lrs_status launch_amp_kernels(lrs_ctx* ctx, const uint64_t* x, int64_t batch, do
 
 }  // namespace
 
+// Scratch of `full` bytes, or of at least `least` where so much cannot be had.  Scratch that is
+// enough for `least` is not given up before a larger one is there (a captured call may address
+// it), and an allocation that has failed is not tried again for as much until the terms' storage
+// changes: such calls reallocate nothing, neither each time nor under capture.
+static lrs_status amp_scratch(lrs_ctx* ctx, size_t full, size_t least, cudaStream_t st) {
+    if (ctx->scratch_bytes >= full) return LRS_OK;
+    const bool keep = ctx->scratch_bytes >= least, tried = ctx->amp_oom != 0 && full >= ctx->amp_oom;
+    if (keep && (tried || lrs_capturing(st))) return LRS_OK;
+    if (!tried) {
+        void* p = keep ? nullptr : ctx->scratch;
+        size_t have = keep ? 0 : ctx->scratch_bytes;
+        const lrs_status rc = lrs_ensure(&p, &have, full, ctx->alloc_limit);
+        if (rc == LRS_OK || !keep) {
+            if (keep) cudaFree(ctx->scratch);
+            ctx->scratch = p;
+            ctx->scratch_bytes = have;
+        }
+        if (rc != LRS_ERR_OOM) return rc;
+        ctx->amp_oom = full;
+        if (keep) return LRS_OK;
+    }
+    void* scr = nullptr;
+    return lrs_scratch(ctx, least, &scr);
+}
+
 // The sliced kernels and the reduction, with scratch for partial sums and their compensations,
-// bounds (err), amplitudes (*amp_out) and records; the string-per-thread kernel where that does
-// not fit, with scratch for no more than its sums.
+// bounds (err), amplitudes (*amp_out) and records: as many of the records as the scratch that
+// could be had holds, and the string-per-thread kernel where that is too few.
 static lrs_status launch_amp_scratch(lrs_ctx* ctx, const uint64_t* x, int64_t batch, const AmpPlan& P, double* out,
                                      double** amp_out, float* err, cudaStream_t st) {
     auto round = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
     const size_t amps = round((size_t)batch * 2 * sizeof(double));
     // bounds and amplitudes have their place in every call, as the sums do
-    size_t sums = amp_partials(ctx, batch), need = 2 * round(sums * sizeof(float2)) + round(sums * sizeof(float)) + amps;
+    const size_t most = amp_partials(ctx, batch), need = 2 * round(most * sizeof(float2)) + round(most * sizeof(float)) + amps;
+    // without records: the sums of this call and what it asked for
+    const size_t sums = (size_t)batch * P.n_tiles;
+    const size_t least = round(sums * sizeof(float2)) + (err ? round(sums * sizeof(float)) : 0) + (amp_out ? amps : 0);
     int64_t records;
     AmpPrep R = amp_records(ctx, &records);
-    void* scr = nullptr;
-    lrs_status rc = lrs_scratch(ctx, need + (size_t)records * R.words * sizeof(uint64_t), &scr);
-    const bool sliced = rc == LRS_OK;
-    if (rc == LRS_ERR_OOM) {
-        sums = (size_t)batch * P.n_tiles;
-        need = round(sums * sizeof(float2)) + (err ? round(sums * sizeof(float)) : 0) + (amp_out ? amps : 0);
-        rc = lrs_scratch(ctx, need, &scr);
-    }
+    const size_t rec_bytes = R.words * sizeof(uint64_t);
+    lrs_status rc = amp_scratch(ctx, need + (size_t)records * rec_bytes, least, st);
     if (rc != LRS_OK) return rc;
-    char* at = (char*)scr;
+    const size_t room = ctx->scratch_bytes > need ? (ctx->scratch_bytes - need) / rec_bytes : 0;
+    if ((size_t)records > room) records = (int64_t)room;
+    R.rl = amp_range(P, ctx->cap, records);
+    char* at = (char*)ctx->scratch;
     auto take = [&](size_t bytes) {
         char* q = at;
         at += round(bytes);
@@ -825,10 +850,9 @@ static lrs_status launch_amp_scratch(lrs_ctx* ctx, const uint64_t* x, int64_t ba
     float2* partial = (float2*)take(sums * sizeof(float2));
     float* magp = err ? (float*)take(sums * sizeof(float)) : nullptr;
     if (amp_out) out = *amp_out = (double*)take(amps);
-    if (!sliced) return launch_amp_kernels(ctx, x, batch, out, partial, P, st, magp, err);
+    if (R.rl == 0) return launch_amp_kernels(ctx, x, batch, out, partial, P, st, magp, err);
     float2* comp = (float2*)take(sums * sizeof(float2));
-    R.rec = (uint64_t*)((char*)scr + need);
-    R.rl = amp_range(P, ctx->cap, records);
+    R.rec = (uint64_t*)((char*)ctx->scratch + need);
     if ((rc = launch_sliced(ctx, x, batch, partial, comp, P, R, magp, st)) != LRS_OK) return rc;
     k_amp_reduce<<<(unsigned)batch, 256, 0, st>>>(partial, magp, P.n_tiles, batch, P.tt, out, err);
     LRS_LAUNCH_CHECK("amplitude reduce kernel");

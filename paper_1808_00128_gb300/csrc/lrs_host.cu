@@ -286,6 +286,7 @@ static void free_terms(lrs_ctx* c) {
     c->F = c->G = c->M = c->glo = c->ghi = c->v = c->s = nullptr;
     c->omega = nullptr; c->coef = nullptr; c->choice = nullptr;
     c->cap = 0; c->chi = 0; c->choice_slots_cap = 0; c->have_terms = false;
+    c->amp_oom = 0;
 }
 
 static void free_chains(lrs_ctx* c) {
@@ -970,6 +971,7 @@ extern "C" lrs_status lrs_debug_limit_alloc(lrs_ctx* c, int64_t bytes) {
     if (!c) return lrs_fail(LRS_ERR_ARG, "ctx is NULL");
     if (bytes < 0) return lrs_fail(LRS_ERR_ARG, "bytes < 0");
     c->alloc_limit = (size_t)bytes;
+    c->amp_oom = 0;
     return LRS_OK;
 }
 

@@ -94,6 +94,7 @@ struct lrs_ctx {
     // scratch for partial sums
     void* scratch = nullptr;
     size_t scratch_bytes = 0;
+    size_t amp_oom = 0;             // least scratch of an amplitude call that could not be had (0: none)
     size_t alloc_limit = 0;         // lrs_debug_limit_alloc: larger buffers fail to allocate (0: none)
     // launch-shape tuning (lrs_set_tuning)
     int64_t tune_amp_bps = 8;       // amplitude: target blocks per SM

@@ -50,3 +50,55 @@ def test_no_steps_on_the_chains_of_a_failed_start(first):
     got = _chains(sim, x0)
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     sim.close()
+
+
+@pytest.mark.parametrize("n", [7, 40, 64])
+def test_amplitudes_without_memory_for_records(n):
+    """lrs_amplitude when the records cannot be had: the string-per-thread kernel in the
+    scratch of its sums, the same bits and bounds, nothing reallocated from call to call,
+    and a capture that replays."""
+    require_cuda()
+    sim = _sim(n, 3000)
+    x = sim.sample_terms(300, seed=4)
+    out = torch.empty((300, 2), dtype=torch.float64, device="cuda")
+    err = torch.empty(300, dtype=torch.float32, device="cuda")
+    want, want_err = sim.amplitude(x, err=err).clone(), err.clone()
+    sim.close()
+    sim = _sim(n, 3000)
+    sim.debug_limit_alloc(300 * 96 * 12 + 1024)      # 96 tiles: a sum and a bound each
+    sim.amplitude(x, out=out, err=err)
+    assert torch.equal(out, want) and torch.equal(err, want_err)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        sim.amplitude(x, out=out)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    few, small = x[:50].contiguous(), torch.empty((50, 2), dtype=torch.float64, device="cuda")
+    for _ in range(3):
+        sim.amplitude(few, out=small)
+        sim.amplitude(x, out=out, err=err)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] == free
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    g.reset()
+    sim.debug_limit_alloc(0)
+    assert torch.equal(sim.amplitude(x), want)
+    sim.close()
+
+
+def test_amplitudes_with_room_for_some_records():
+    """Scratch left by a norm estimate that holds some of the records: launches over parts of
+    every tile, the same bits."""
+    require_cuda()
+    sim = _sim(40, 20000)
+    x = sim.sample_terms(1500, seed=4)
+    want = sim.amplitude(x).clone()
+    sim.close()
+    sim = _sim(40, 20000)
+    sim.norm_estimate(4450, seed=1)                  # about 32.7 MB; 34.5 for all records
+    sim.debug_limit_alloc(1000)
+    assert torch.equal(sim.amplitude(x), want)
+    sim.close()
