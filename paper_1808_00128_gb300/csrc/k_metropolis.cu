@@ -864,9 +864,11 @@ static lrs_status enqueue_steps(lrs_ctx* ctx, int64_t t0, int64_t count, float2*
 }
 
 // One CUDA graph holding LRS_MC_GRAPH_STEPS steps followed by step0 += steps;
-// rebuilt whenever the buffers it was captured with change.
+// rebuilt whenever one of the buffers it was captured with changes: each of them by its own
+// address, as any may come back to an old one alone (fewer chains after more reallocate cx, cp and
+// pend, and may find the states and planes where they were).
 static lrs_status mc_graph(lrs_ctx* ctx, float2* partial, int32_t* jprop, cudaGraphExec_t* out) {
-    const void* key[6] = {partial, jprop, ctx->Q, ctx->mc_planes,
+    const void* key[9] = {partial, jprop, ctx->Q, ctx->mc_planes, ctx->cx, ctx->cp, ctx->pend,
                           (void*)(intptr_t)(((ctx->n_chains * 128 + ctx->tune_mc_cg) * 8 + ctx->tune_mc_stages) * 4 +
                                             ctx->tune_mc_lookahead),
                           (void*)(intptr_t)ctx->cap};

@@ -127,7 +127,7 @@ struct lrs_ctx {
     int* mc_err_h = nullptr;        // mapped host [2]: a propose kernel gave up waiting; test request
     int* mc_err_d = nullptr;        // its device address
     void* mc_exec = nullptr;        // cudaGraphExec_t of LRS_MC_GRAPH_STEPS steps
-    const void* mc_key[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    const void* mc_key[9] = {};
     void* cap_stream = nullptr;     // cudaStream_t used for graph capture
     // learned-proposal Metropolis-Hastings buffers
     uint64_t* ybuf = nullptr;       // [chain] proposals

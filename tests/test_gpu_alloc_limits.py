@@ -102,3 +102,27 @@ def test_amplitudes_with_room_for_some_records():
     sim.debug_limit_alloc(1000)
     assert torch.equal(sim.amplitude(x), want)
     sim.close()
+
+
+def test_chain_counts_up_and_down_between_graph_replays():
+    """Steps replayed from the context's graph (16 at a time) after the chains' buffers moved: the
+    chains of a context that never held another number."""
+    require_cuda()
+    sim = _sim()
+    x0 = sim.sample_terms(700, seed=2)
+    want = {}
+    for c in (100, 200, 700):
+        one = _sim()
+        want[c] = _chains(one, x0[:c].contiguous(), steps=33)
+        one.close()
+    for c in (100, 200, 100, 700, 100, 200, 700, 100):
+        got = _chains(sim, x0[:c].contiguous(), steps=33)
+        assert torch.equal(got[0], want[c][0]) and torch.equal(got[1], want[c][1]), c
+    # new storage of the terms, and back
+    low = lrstab.lower_circuit(40, workloads.random_clifford_t(40, 320, 12, 5))
+    for chi in (9000, 3000):
+        sim.init_terms(low, chi, mode="sparsify", seed=5)
+        sim.apply_clifford(low.gates)
+        got = _chains(sim, x0[:100].contiguous(), steps=33)
+    assert torch.equal(got[0], want[100][0]) and torch.equal(got[1], want[100][1])
+    sim.close()
