@@ -37,6 +37,7 @@ constexpr int NRM_WINDOW = 16;   // rows searched for the pivot row's partner
 constexpr int NRM_STRIDE = 66;   // words per row of A in shared memory; column 64 and row n are zero
 constexpr int NRM_END = 10;      // variables left to the per-form elimination
 constexpr int NRM_SYNC = 4;      // terms between the barriers of a block
+constexpr int NRM_VEC = 88;      // entries of the shared vectors: past the last row that a step reads (stage)
 constexpr int NRM_CHUNK = 32;    // terms whose values a cooperating block collects at a time
 
 // Record of a term: `rows` words of bit rows, then eight header words, then the pivots as
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(256) k_norm_prep(TermsView T, NormPrep P) {
 // Work area of a warp in shared memory.
 struct NormWarp {
     uint4 pa[80];            // per column: pivot row, second row, linear planes
-    uint2 pb[80];            // per column: the two vectors of a rank-2 update
+    uint2 pb[NRM_VEC];       // per column: the two vectors of a rank-2 update
     uint32_t off[80];        // first word of row (natural index of the variable) in A
     union {
         uint32_t rows[NRM_END][32];   // last rows, one form per lane
@@ -266,6 +267,7 @@ struct NormWarp {
     uint32_t diag[2][16];
     uint64_t rec[2][80];     // record of this term and the next
 };
+static_assert(sizeof(NormWarp) % 16 == 0, "the warps' areas follow one another");
 
 // c ^ (a & b), one instruction (left to itself the compiler forms a three-way XOR of two
 // ANDs where two of these do)
@@ -452,9 +454,12 @@ __device__ __forceinline__ void finish_many(Forms<NR, NC>& Z, int lane, uint32_t
     finish_long<R, C>(S, L, Z.a, Z.m - Z.a, lane, s0, s1, z0, z1, e);
 }
 
-// Sliced steps while more than LOW variables are left, R rows at most.
+// Sliced steps while more than LOW variables are left, R rows at most.  A step starts at
+// a <= NR - LOW - 2 (a even, m <= NR) and reads R entries of the shared vectors from there; with one
+// column a lane from a mod 32.
 template <int R, int C, int LOW, int NR, int NC>
 __device__ __forceinline__ bool stage(Forms<NR, NC>& Z, NormWarp& W, int lane, int pos) {
+    static_assert((C == 1 ? 30 : NR - LOW - 2) + R <= NRM_VEC, "a step reads past the shared vectors");
 #pragma unroll 1
     while (Z.m - Z.a > LOW)
         if (!eliminate_pair<R, C>(Z, W, lane, pos)) return false;
@@ -778,9 +783,10 @@ __global__ void __launch_bounds__(32 * norm_warps(NR), 1)
         sD[i] = c < n ? P.ad[(g * 2 + r) * 64 + c] : 0u;
     }
     NormWarp& W = sW[warp];
-    for (int i = lane; i < 80; i += 32) {
-        W.pa[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = lane; i < NRM_VEC; i += 32) {
         W.pb[i] = make_uint2(0u, 0u);
+        if (i >= 80) break;
+        W.pa[i] = make_uint4(0u, 0u, 0u, 0u);
         W.off[i] = (uint32_t)(n * NRM_STRIDE);
     }
     const int64_t tile = COOP ? tb : tb * NW + warp;
