@@ -553,8 +553,12 @@ __global__ void __launch_bounds__(AS_TPB, 2) k_amp_sliced(AmpPrep P, int n, uint
     for (int k = 0; k < 4; ++k) {
         sum[k] = nc[k] = 0;
         mag[k] = 0.f;
-        const int64_t i = (xb * wl + l) * 32 + 4 * warp + k;
-        if (P.r0 > 0 && tile < n_tiles && i < batch) {   // as the launch before left them
+    }
+    if (P.r0 > 0) {   // as the launch before left them
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t i = (xb * wl + l) * 32 + 4 * warp + k;
+            if (tile >= n_tiles || i >= batch) continue;
             sum[k] = reinterpret_cast<const uint64_t*>(partial)[i * n_tiles + tile];
             nc[k] = reinterpret_cast<const uint64_t*>(comp)[i * n_tiles + tile];
             if (ERR) mag[k] = magp[i * n_tiles + tile];
