@@ -688,8 +688,9 @@ lrs_status launch_sliced_t(lrs_ctx* ctx, const AmpPrep& R, const uint64_t* x, in
     const size_t smem = 8192 + (size_t)NC * 8192 +
                         (size_t)AS_TERMS * 32 * (3 * sizeof(uint32_t) + sizeof(float2) + (magp ? sizeof(float) : 0));
     const auto kernel = magp ? k_amp_sliced<NC, true> : k_amp_sliced<NC, false>;
-    if (!lrs_capturing(st))
-        LRS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // also under capture (it is no stream operation): the call that sized the scratch may have been
+    // one with the other choice of bounds
+    LRS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int64_t G = 32 / wl, tgroups = (P.n_tiles + G - 1) / G;
     const int64_t blocks = tgroups * ((batch + 32 * wl - 1) / (32 * wl));
     if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "amplitude grid too large");

@@ -70,3 +70,26 @@ def test_several_launches_equal_the_string_kernel(n, chi):
         mag = want.norm(dim=1)
         assert bool((err >= 0).all()) and bool((err[mag > 0] > 0).all())
     sim.close()
+
+
+@pytest.mark.parametrize("n", [19, 31, 45, 53])
+def test_capture_after_a_call_of_the_other_kind(n):
+    """A call with bounds sizes the scratch for one without: the capture of the latter, whose
+    kernel has then not run, and the other way round (at widths that no other test of this
+    file runs)."""
+    require_cuda()
+    for bounds in (True, False):
+        sim = _sim(n + bounds, 500)
+        x = _strings(sim, 200)
+        want, out = (torch.empty((200, 2), dtype=torch.float64, device="cuda") for _ in range(2))
+        err = torch.empty(200, dtype=torch.float32, device="cuda")
+        sim.amplitude(x, out=want, err=err if bounds else None)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            sim.amplitude(x, out=out, err=None if bounds else err)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        g.reset()
+        sim.close()
