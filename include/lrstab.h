@@ -352,7 +352,11 @@ lrs_status lrs_sample_terms(lrs_ctx* ctx, int64_t count, uint64_t seed, uint64_t
 /* Start n_chains chains at x_dev[c]: computes the phase and the constraints'
  * syndromes of every (chain, term) at x and P(x) = |<x|psi>|^2.  Needs n <= 62.
  * Storage, owned by the context: (4 + n, rounded up to even) bits per (chain, term)
- * and (1.5 n^2 + 3 n) bits + 8 bytes per term for the terms' bit-planes.
+ * and (1.5 n^2 + 3 n) bits + 8 bytes per term for the terms' bit-planes.  Where that
+ * cannot be allocated and the chains are few (a 12-byte, for n > 40 16-byte, state per
+ * (chain, term) would take less: fewer than about 50), the chains keep their strings
+ * only and every step evaluates the amplitudes of its proposals: the same draws and
+ * the same test, slower.
  * Errors: LRS_ERR_ARG, LRS_ERR_STATE, LRS_ERR_UNSUPPORTED (n > 62), LRS_ERR_OOM. */
 lrs_status lrs_chains_init(lrs_ctx* ctx, int64_t n_chains, const uint64_t* x_dev, void* stream);
 

@@ -715,6 +715,16 @@ __global__ void k_metro_accept_amp(const double* __restrict__ amp, int64_t C, ui
     if (trace) trace[c] = cx[c];
 }
 
+// Chains without states (ctx->mc_direct): the strings that step `step` proposes.
+__global__ void k_mc_strings(int64_t C, uint64_t seed, int64_t step, int n, const uint64_t* __restrict__ cx,
+                             uint64_t* __restrict__ y, int32_t* __restrict__ jprop) {
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= C) return;
+    const int j = draw_j(seed, c, step, n);
+    jprop[c] = j;
+    y[c] = cx[c] ^ bit64(j);
+}
+
 __global__ void k_chains_set_prob(const double* __restrict__ amp, int64_t C, double* cp) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c < C) cp[c] = amp[2 * c] * amp[2 * c] + amp[2 * c + 1] * amp[2 * c + 1];
@@ -771,14 +781,16 @@ static int mc_columns(int64_t cols) {
 
 // States and P(x) of the chains at strings x.
 static lrs_status mc_start(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) {
-    McView V;
-    mc_layout(ctx, &V);
     const int64_t C = ctx->n_chains;
-    const int tbx = mc_columns(V.cols), nsub = MC_TPB / tbx;
-    const int64_t cblocks = (C + nsub - 1) / nsub, blocks = (V.cols + tbx - 1) / tbx * cblocks;
-    if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "chain start grid too large");
-    k_mc_start<<<(unsigned)blocks, MC_TPB, 0, st>>>(V, C, (uint2*)ctx->Q, x, ctx->nmask, tbx, cblocks);
-    LRS_LAUNCH_CHECK("chain start kernel");
+    if (!ctx->mc_direct) {
+        McView V;
+        mc_layout(ctx, &V);
+        const int tbx = mc_columns(V.cols), nsub = MC_TPB / tbx;
+        const int64_t cblocks = (C + nsub - 1) / nsub, blocks = (V.cols + tbx - 1) / tbx * cblocks;
+        if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "chain start grid too large");
+        k_mc_start<<<(unsigned)blocks, MC_TPB, 0, st>>>(V, C, (uint2*)ctx->Q, x, ctx->nmask, tbx, cblocks);
+        LRS_LAUNCH_CHECK("chain start kernel");
+    }
     double* amp = nullptr;
     lrs_status rc = launch_amplitude_start(ctx, x, C, &amp, st);
     if (rc != LRS_OK) return rc;
@@ -789,6 +801,7 @@ static lrs_status mc_start(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) {
 
 lrs_status launch_chains_init(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) {
     // the planes of the current terms, then the chains' states and probabilities
+    if (ctx->mc_direct) return mc_start(ctx, x, st);
     McView V;
     mc_layout(ctx, &V);
     const size_t smem = (size_t)ctx->n * 256 * sizeof(uint64_t);
@@ -914,9 +927,42 @@ lrs_status mc_flags(lrs_ctx* ctx) {
     return LRS_OK;
 }
 
+// Strings that every chain without states proposes (ybuf, their flips in jbuf).
+static lrs_status mc_propose_strings(lrs_ctx* ctx, uint64_t seed, int64_t step, cudaStream_t st) {
+    const int64_t C = ctx->n_chains;
+    lrs_status rc = lrs_ensure((void**)&ctx->jbuf, &ctx->jbuf_bytes, (size_t)C * sizeof(int32_t));
+    if (rc != LRS_OK) return rc;
+    k_mc_strings<<<(unsigned)((C + 127) / 128), 128, 0, st>>>(C, seed, step, ctx->n, ctx->cx, ctx->ybuf, ctx->jbuf);
+    LRS_LAUNCH_CHECK("proposal strings kernel");
+    return LRS_OK;
+}
+
+// Steps of chains without states: the amplitudes of the proposed strings over all terms, the same
+// draws and the same FP64 test.  No memory per (chain, term), at an amplitude call per step
+// (41 strings of 2^24 terms at n = 40: 25 ms).
+static lrs_status mc_direct_steps(lrs_ctx* ctx, int64_t steps, uint64_t seed, int64_t step0, uint64_t* trace,
+                                  cudaStream_t st) {
+    const int64_t C = ctx->n_chains;
+    for (int64_t t = 0; t < steps; ++t) {
+        double* amp = nullptr;
+        lrs_status rc = mc_propose_strings(ctx, seed, step0 + t, st);
+        if (rc == LRS_OK) rc = launch_amplitude_start(ctx, ctx->ybuf, C, &amp, st);
+        if (rc == LRS_OK) rc = launch_metropolis_accept(ctx, amp, seed, step0 + t, trace ? trace + t * C : nullptr, st);
+        if (rc != LRS_OK) return rc;
+    }
+    return LRS_OK;
+}
+
 lrs_status launch_metropolis(lrs_ctx* ctx, int64_t steps, uint64_t seed, int64_t step0,
                              uint64_t* x_out, double* p_out, uint64_t* trace, cudaStream_t st) {
     const int64_t C = ctx->n_chains;
+    if (ctx->mc_direct) {
+        const lrs_status rd = mc_direct_steps(ctx, steps, seed, step0, trace, st);
+        if (rd != LRS_OK) return rd;
+        k_metro_out<<<(unsigned)((C + 127) / 128), 128, 0, st>>>(C, ctx->cx, ctx->cp, x_out, p_out);
+        LRS_LAUNCH_CHECK("metropolis out kernel");
+        return LRS_OK;
+    }
     const int64_t n_tiles = ctx->cap / MC_TERMS;
     void* scr = nullptr;
     // partial sums: three per chain and tile for two-step passes; proposals j_t, j_{t+1}
@@ -958,14 +1004,16 @@ lrs_status launch_metropolis(lrs_ctx* ctx, int64_t steps, uint64_t seed, int64_t
 // this context's terms (the pending flip of the previous step is applied to Q first).
 lrs_status launch_metropolis_propose(lrs_ctx* ctx, uint64_t seed, int64_t step, double* amp, cudaStream_t st) {
     const int64_t C = ctx->n_chains;
+    lrs_status rc;
+    if (ctx->mc_direct) {
+        if ((rc = mc_propose_strings(ctx, seed, step, st)) != LRS_OK) return rc;
+        return launch_amplitude(ctx, ctx->ybuf, C, amp, nullptr, st);
+    }
     const int64_t n_tiles = ctx->cap / MC_TERMS;
     void* scr = nullptr;
-    lrs_status rc = lrs_scratch(ctx, (size_t)C * n_tiles * sizeof(float2), &scr);
-    if (rc != LRS_OK) return rc;
+    if ((rc = lrs_scratch(ctx, (size_t)C * n_tiles * sizeof(float2), &scr)) != LRS_OK) return rc;
     if (!ctx->mc_par) LRS_CUDA(cudaMalloc(&ctx->mc_par, sizeof(McParams)));
-    size_t have = ctx->jbuf_bytes;
-    if ((rc = lrs_ensure((void**)&ctx->jbuf, &have, (size_t)C * sizeof(int32_t))) != LRS_OK) return rc;
-    ctx->jbuf_bytes = have;
+    if ((rc = lrs_ensure((void**)&ctx->jbuf, &ctx->jbuf_bytes, (size_t)C * sizeof(int32_t))) != LRS_OK) return rc;
     if ((rc = mc_flags(ctx)) != LRS_OK) return rc;
     if (*(volatile int*)ctx->mc_err_h) {
         *(volatile int*)ctx->mc_err_h = 0;
@@ -998,22 +1046,27 @@ lrs_status launch_chains_set_prob(lrs_ctx* ctx, const double* amp, cudaStream_t 
     return LRS_OK;
 }
 
+lrs_status mh_buffers(lrs_ctx* ctx, int64_t C) {
+    if (C <= ctx->mh_cap) return LRS_OK;
+    cudaFree(ctx->ybuf); cudaFree(ctx->lqy); cudaFree(ctx->lqx); cudaFree(ctx->ampy);
+    ctx->ybuf = nullptr; ctx->lqy = nullptr; ctx->lqx = nullptr; ctx->ampy = nullptr;
+    ctx->mh_cap = 0;
+    LRS_CUDA(cudaMalloc(&ctx->ybuf, (size_t)C * sizeof(uint64_t)));
+    LRS_CUDA(cudaMalloc(&ctx->lqy, (size_t)C * sizeof(float)));
+    LRS_CUDA(cudaMalloc(&ctx->lqx, (size_t)C * sizeof(float)));
+    LRS_CUDA(cudaMalloc(&ctx->ampy, (size_t)C * 2 * sizeof(double)));
+    ctx->mh_cap = C;
+    return LRS_OK;
+}
+
 lrs_status launch_metropolis_learned(lrs_ctx* ctx, lrs_mlp* mlp, int64_t steps, uint64_t seed, int64_t step0,
                                      uint64_t* x_out, double* p_out, uint64_t* trace, int64_t* accepts,
                                      cudaStream_t st) {
     const int64_t C = ctx->n_chains;
-    if (C > ctx->mh_cap) {
-        cudaFree(ctx->ybuf); cudaFree(ctx->lqy); cudaFree(ctx->lqx); cudaFree(ctx->ampy);
-        ctx->ybuf = nullptr; ctx->lqy = nullptr; ctx->lqx = nullptr; ctx->ampy = nullptr;
-        ctx->mh_cap = 0;
-        LRS_CUDA(cudaMalloc(&ctx->ybuf, (size_t)C * sizeof(uint64_t)));
-        LRS_CUDA(cudaMalloc(&ctx->lqy, (size_t)C * sizeof(float)));
-        LRS_CUDA(cudaMalloc(&ctx->lqx, (size_t)C * sizeof(float)));
-        LRS_CUDA(cudaMalloc(&ctx->ampy, (size_t)C * 2 * sizeof(double)));
-        ctx->mh_cap = C;
-    }
+    lrs_status rc = mh_buffers(ctx, C);
+    if (rc != LRS_OK) return rc;
     // log q of the current states under the current network
-    lrs_status rc = lrs_mlp_forward(mlp, ctx->cx, C, nullptr, ctx->lqx, st);
+    rc = lrs_mlp_forward(mlp, ctx->cx, C, nullptr, ctx->lqx, st);
     if (rc != LRS_OK) return rc;
     for (int64_t t = 0; t < steps; ++t) {
         const int64_t step = step0 + t;

@@ -287,6 +287,7 @@ static void free_terms(lrs_ctx* c) {
     c->omega = nullptr; c->coef = nullptr; c->choice = nullptr;
     c->cap = 0; c->chi = 0; c->choice_slots_cap = 0; c->have_terms = false;
     c->amp_oom = 0;
+    c->mc_oom = 0;
 }
 
 static void free_chains(lrs_ctx* c) {
@@ -881,10 +882,29 @@ extern "C" lrs_status lrs_chains_init(lrs_ctx* c, int64_t n_chains, const uint64
     if (n_chains > 65535) return lrs_fail(LRS_ERR_ARG, "at most 65535 chains");
     LRS_CUDA(cudaSetDevice(c->device));
     c->n_chains = 0;   // until every buffer is there and set: no steps on the chains of a failed call
-    lrs_status rc = lrs_ensure((void**)&c->Q, &c->Q_bytes, mc_state_bytes(c, n_chains), c->alloc_limit);
-    if (rc != LRS_OK) return rc;
-    rc = lrs_ensure(&c->mc_planes, &c->mc_planes_bytes, mc_planes_bytes(c), c->alloc_limit);
-    if (rc != LRS_OK) return rc;
+    // The planes take as much for one chain as for many.  Chains so few that a Pauli pair
+    // i^mu X(u) Z(w) per (chain, term), 12 or 16 bytes, would take less (about 50 at n = 40 or 50)
+    // do without planes and states where these cannot be had; and an allocation that has
+    // failed is not tried again for as much until the terms' storage changes.
+    const size_t states = mc_state_bytes(c, n_chains), planes = mc_planes_bytes(c);
+    const bool few = (size_t)n_chains * c->cap * (c->n <= 40 ? 12 : 16) < planes + states;
+    lrs_status rc = LRS_OK;
+    c->mc_direct = few && c->mc_oom != 0 && planes + states >= c->mc_oom &&
+                   (c->Q_bytes < states || c->mc_planes_bytes < planes);
+    if (!c->mc_direct) {
+        rc = lrs_ensure((void**)&c->Q, &c->Q_bytes, states, c->alloc_limit);
+        if (rc == LRS_OK) rc = lrs_ensure(&c->mc_planes, &c->mc_planes_bytes, planes, c->alloc_limit);
+        if (rc == LRS_ERR_OOM && few) {
+            cudaFree(c->Q); cudaFree(c->mc_planes);
+            c->Q = nullptr; c->mc_planes = nullptr;
+            c->Q_bytes = c->mc_planes_bytes = 0;
+            c->mc_oom = planes + states;
+            c->mc_direct = true;
+            rc = LRS_OK;
+        }
+        if (rc != LRS_OK) return rc;
+    }
+    if (c->mc_direct && (rc = mh_buffers(c, n_chains)) != LRS_OK) return rc;
     if (n_chains > c->chains_cap) {
         cudaFree(c->cx); cudaFree(c->cp); cudaFree(c->pend);
         c->cx = nullptr; c->cp = nullptr; c->pend = nullptr;
@@ -972,6 +992,7 @@ extern "C" lrs_status lrs_debug_limit_alloc(lrs_ctx* c, int64_t bytes) {
     if (bytes < 0) return lrs_fail(LRS_ERR_ARG, "bytes < 0");
     c->alloc_limit = (size_t)bytes;
     c->amp_oom = 0;
+    c->mc_oom = 0;
     return LRS_OK;
 }
 

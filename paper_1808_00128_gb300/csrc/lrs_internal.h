@@ -118,6 +118,8 @@ struct lrs_ctx {
     size_t Q_bytes = 0;
     void* mc_planes = nullptr;      // bit-planes of the terms, made by lrs_chains_init
     size_t mc_planes_bytes = 0;
+    bool mc_direct = false;         // neither could be had: every step evaluates its strings' amplitudes
+    size_t mc_oom = 0;              // least bytes of both that could not be had (0: none)
     uint64_t* cx = nullptr;         // [chain] current x
     double* cp = nullptr;           // [chain] P(x) (unnormalised)
     int32_t* pend = nullptr;        // [2][chain] pending accepted flips, committed in order (-1 none)
@@ -193,6 +195,8 @@ lrs_status launch_norm_eta(const double* ov, int64_t L, double* eta, cudaStream_
 lrs_status launch_sample_terms(lrs_ctx* ctx, int64_t count, uint64_t seed, uint64_t* x,
                                int64_t* alpha, cudaStream_t st);
 lrs_status launch_chains_init(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st);
+// Buffers of ctx->n_chains proposals (strings, log q, amplitudes).
+lrs_status mh_buffers(lrs_ctx* ctx, int64_t chains);
 // bytes of the chains' buffers (device memory is the caller's business)
 size_t mc_planes_bytes(const lrs_ctx* ctx);
 size_t mc_state_bytes(const lrs_ctx* ctx, int64_t chains);

@@ -1,6 +1,7 @@
 """Calls whose device buffers cannot be allocated (lrs_debug_limit_alloc makes the
 allocations fail on the host): they report it, and leave nothing behind that a later call would
 run on."""
+import numpy as np
 import pytest
 import torch
 
@@ -126,3 +127,73 @@ def test_chain_counts_up_and_down_between_graph_replays():
         got = _chains(sim, x0[:100].contiguous(), steps=33)
     assert torch.equal(got[0], want[100][0]) and torch.equal(got[1], want[100][1])
     sim.close()
+
+
+@pytest.mark.parametrize("n", [40, 55])
+def test_few_chains_without_memory_for_their_planes(n):
+    """The steps of few chains whose planes cannot be had: the strings and, to the rounding of the
+    sums, the probabilities of the chains that have them; through the calls of a sharded step
+    and under capture too, nothing reallocated."""
+    require_cuda()
+    sim = _sim(n)
+    x0 = sim.sample_terms(8, seed=2)
+
+    def trace(steps, step0=0):
+        tr = torch.empty((steps, 8), dtype=torch.int64, device="cuda")
+        p = torch.empty(8, dtype=torch.float64, device="cuda")
+        sim.metropolis(steps, seed=8, step0=step0, trace=tr, p_out=p)
+        return tr, p
+
+    sim.chains_init(x0)
+    want, want_p = trace(40)
+    assert int((want[-1] != x0).sum()) > 0
+    sim.close()
+    sim = _sim(n)
+    sim.debug_limit_alloc(100_000)
+    sim.chains_init(x0)
+    a, _ = trace(15)
+    row = torch.empty(8, dtype=torch.int64, device="cuda")
+    for step in (15, 16):
+        amp = sim.metropolis_propose(8, step)
+        sim.metropolis_accept(amp, 8, step, trace=row)
+        a = torch.cat([a, row[None]])
+    b, p = trace(23, 17)
+    assert torch.equal(torch.cat([a, b]), want)
+    assert bool(((p - want_p).abs() <= 1e-5 * torch.clamp(want_p, min=2.0 ** -n)).all())
+    with pytest.raises(lrstab.LrsError) as e:        # not for many
+        sim.chains_init(sim.sample_terms(200, seed=2))
+    assert e.value.status == OOM
+    sim.chains_init(x0)
+    x, p = torch.empty_like(x0), torch.empty_like(p)
+    sim.metropolis(40, seed=8, x_out=x, p_out=p)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        sim.chains_init(x0)
+        sim.metropolis(40, seed=8, x_out=x, p_out=p)
+    x.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(x, want[-1])
+    g.reset()
+    sim.close()
+
+
+def test_learned_steps_of_chains_without_planes():
+    require_cuda()
+    n = 40
+    net = lrstab.MLP(n, 64)
+    net.set_params(dict(W1=np.zeros((64, n)), b1=np.zeros(64), W2=np.zeros((64, 64)), b2=np.zeros(64),
+                        W3=np.zeros((n, 64)), b3=np.zeros(n)))
+    out = []
+    for limit in (0, 100_000):
+        sim = _sim(n)
+        x0 = sim.sample_terms(8, seed=2)
+        sim.debug_limit_alloc(limit)
+        sim.chains_init(x0)
+        x = torch.empty_like(x0)
+        lrstab.metropolis_learned(sim, net, 3, seed=4)
+        sim.metropolis(9, seed=8, x_out=x)
+        out.append(x)
+        sim.close()
+    net.close()
+    assert torch.equal(*out)
