@@ -40,8 +40,9 @@ constexpr int NRM_SYNC = 4;      // terms between the barriers of a block
 constexpr int NRM_VEC = 88;      // entries of the shared vectors: past the last row that a step reads (stage)
 constexpr int NRM_CHUNK = 32;    // terms whose values a cooperating block collects at a time
 
-// Record of a term: `rows` words of bit rows, then eight header words, then the pivots as
-// bytes.  Rows 0..m-1: the restricted form of J between free variables (bit k of row k:
+// Record of a term: `rows` words of bit rows, then six header words, then the pivots as bytes
+// (14 words beside the rows: near the memory limit the scratch of a call is mostly these
+// records).  Rows 0..m-1: the restricted form of J between free variables (bit k of row k:
 // its odd diagonal).  Rows from m on: h of every constraint (n - m of them); or, for a term
 // with few free variables (norm_basis), the y' of every free variable (m vectors over the
 // n qubits) and the constant vector c.
@@ -50,7 +51,7 @@ struct NormPrep {
     int words, rows;
     uint32_t *A, *ad;       // [group][n][64] and [group][2][64]: entries, diagonal planes
 };
-enum { REC_FREE = 0, REC_LO, REC_HI, REC_CONST, REC_INFO, REC_COEF, REC_PIV = 8, REC_HEAD = 16 };
+enum { REC_FREE = 0, REC_LO, REC_HI, REC_CONST, REC_INFO, REC_COEF, REC_PIV, REC_HEAD = REC_PIV + 8 };
 
 // Few free variables: q_A is evaluated on the basis (m + 1 matrix-vector products and
 // m^2 / 2 dot products over the lanes) instead of folding n - m constraints one by one, whose

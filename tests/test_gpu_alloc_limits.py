@@ -197,3 +197,17 @@ def test_learned_steps_of_chains_without_planes():
         sim.close()
     net.close()
     assert torch.equal(*out)
+
+
+@pytest.mark.parametrize("n", [9, 40, 63, 64])
+def test_norm_estimate_in_fifteen_words_and_a_row_per_term(n):
+    """Scratch of lrs_norm_estimate: the partial sums, n + 15 words a term and n + 2 a state."""
+    require_cuda()
+    sim = _sim(n, 100_000)
+    want = sim.norm_estimate(96, seed=3).clone()
+    sim.close()
+    sim = _sim(n, 100_000)
+    cap, tiles = 100_096, 1564                       # tiles of 64 terms
+    sim.debug_limit_alloc((96 * tiles + 31) // 32 * 32 * 8 + 8 * (cap * (n + 15) + 96 * (n + 2)))
+    assert torch.equal(sim.norm_estimate(96, seed=3), want)
+    sim.close()
