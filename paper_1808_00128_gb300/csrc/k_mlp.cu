@@ -20,7 +20,7 @@
 typedef __nv_bfloat16 bf16;
 
 struct lrs_mlp {
-    int device = 0;
+    int device = 0, sm_count = 0;
     int n = 0, NP = 64, H = 0;
     // FP32 master parameters and AdamW moments (device)
     float *W1 = nullptr, *b1 = nullptr, *W2 = nullptr, *b2 = nullptr, *W3 = nullptr, *b3 = nullptr;
@@ -972,13 +972,63 @@ __global__ void k_logq(const float* __restrict__ logits, const uint64_t* __restr
 }
 
 // ---- autoregressive sampling ---------------------------------------------------------------
+// Two routes (sample_in_one says which): a product and a launch pair per bit, or one launch.
+//
+// A product per bit: the tensor cores form the whole second layer n times, n times the work
+// needed, but each at their rate and with W2 read once per tile of rows.
+// Z1 [M][H] fp32 starts at b1; H1 = bf16(relu(Z1)); y = 0, logq = 0.
+__global__ void k_sample_init(const float* __restrict__ b1, int Mp, int H, int count, float* Z1, bf16* H1,
+                              uint64_t* y, float* logq) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < (int64_t)Mp * H) {
+        const float z = b1[i % H];
+        Z1[i] = z;
+        H1[i] = __float2bfloat16_rn(fmaxf(z, 0.f));
+    }
+    if (i < count) {
+        y[i] = 0ull;
+        logq[i] = 0.f;
+    }
+}
+
+// bit i of every sample: logit_i = H2[r] . W3b[i] + b3[i]; y_i = [u < sigmoid];
+// then Z1 += y_i W1b[:, i] and H1 = bf16(relu(Z1)).  One warp per row.
+__global__ void k_sample_bit(const bf16* __restrict__ H2, const bf16* __restrict__ W3b,
+                             const float* __restrict__ b3, const bf16* __restrict__ W1b, int M, int H,
+                             int NP, int i, uint64_t seed, int64_t sid0, float* Z1, bf16* H1, uint64_t* y,
+                             float* logq) {
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (warp >= M) return;
+    const int r = warp;
+    float s = 0.f;
+    for (int k = lane; k < H; k += 32)
+        s += __bfloat162float(H2[(size_t)r * H + k]) * __bfloat162float(W3b[(size_t)i * H + k]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    const float z = s + b3[i];
+    const float p = 1.f / (1.f + expf(-z));
+    // uniform draw: rand64(seed, 2^40 + sample id, bit i)
+    const double u = sm64_unit(sm64_at(sm64_key(seed, (1ull << 40) + (uint64_t)(sid0 + r)), (uint64_t)i));
+    const int bit = (float)u < p ? 1 : 0;
+    if (lane == 0) {
+        if (bit) y[r] |= 1ull << i;
+        logq[r] += -(fmaxf(z, 0.f) + log1pf(expf(-fabsf(z))) - (float)bit * z);
+    }
+    if (bit) {
+        for (int k = lane; k < H; k += 32) {
+            const float zz = Z1[(size_t)r * H + k] + __bfloat162float(W1b[(size_t)k * NP + i]);
+            Z1[(size_t)r * H + k] = zz;
+            H1[(size_t)r * H + k] = __float2bfloat16_rn(fmaxf(zz, 0.f));
+        }
+    }
+}
+
 // Sampling in one launch.  The masks make hidden units of degree d (k = d - 1 mod n - 1) final
 // once bits 0 .. d - 1 are drawn, and bit i reads units of degree <= i only, so each unit of
 // either layer is evaluated once per sample: before bit i the units of degree i (H1 from the
 // bits, H2 from H1), then the logit.  A block draws all n bits of R rows with both layers'
 // activations in shared memory; H1 and H2 of later units stay zero, as their masked weights
-// are.  (A product of the whole H x H layer and a launch pair per bit took n times the work: about
-// 370 us for 1024 samples at n = 20, H = 512, against 102.)
+// are.  1024 samples at n = 20, H = 512: 112 us, with a product per bit 395.
 // Bounded by latency: three barriers a bit, the weights of a bit loaded one phase ahead;
 // activations are kept as FP32 (of their BF16 roundings), so that the products are packed FP32
 // pairs without conversions.
@@ -1275,8 +1325,11 @@ extern "C" lrs_status lrs_mlp_create(int32_t device, int32_t n, int32_t hidden, 
     if (n < 2 || n > 64) return lrs_fail(LRS_ERR_ARG, "MADE needs 2 <= n <= 64 (got %d)", n);
     if (hidden < 64 || hidden > 4096 || hidden % 64) return lrs_fail(LRS_ERR_ARG, "hidden must be a multiple of 64 in 64..4096");
     LRS_CUDA(cudaSetDevice(device));
+    int sms = 0;
+    LRS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
     lrs_mlp* m = new lrs_mlp();
     m->device = device;
+    m->sm_count = sms;
     m->n = n;
     m->H = hidden;
     const int64_t H = hidden;
@@ -1487,6 +1540,30 @@ extern "C" lrs_status lrs_mlp_train_step(lrs_mlp* m, const uint64_t* x, int64_t 
     return refresh_bf16(m, st);
 }
 
+// Rows per block of k_sample: the fewest whose blocks, one per SM, all run at once; with more
+// samples eight, so that W2, which every block reads, is read least often (four where the
+// activations of eight rows, 64 H bytes, do not fit).
+static int sample_rows(const lrs_mlp* m, int M) {
+    if (M <= 2 * m->sm_count) return 2;
+    return M <= 4 * m->sm_count || (size_t)64 * m->H > SMP_SMEM ? 4 : 8;
+}
+
+// One launch, or a product per bit?  The launch does the H x H layer once per sample on the FP32
+// pipe, a block's rows in waves over the SMs; the products do it n times at the tensor cores'
+// rate, with a floor per bit.  So the launch wins up to a wave or a few, and loses by up to 25
+// times for few qubits, wide layers and many samples.  Both sides as fitted to 492 measured times, n = 2..64, H = 64..4096, 1..65536 samples
+// (us; the choice is within 11% of the faster side on every one):
+//   n = 20, H = 512:    1024 samples 112 (products 395), 4096 373 (487), 65536 4965 (3240)
+//   n = 50, H = 512:    1024 201 (951), 16384 2548 (2693), 65536 9886 (7933)
+//   n = 4, H = 4096:    64 754 (310), 16384 33783 (2483)
+static bool sample_in_one(const lrs_mlp* m, int M) {
+    const double n = m->n, H = m->H, R = sample_rows(m, M);
+    const int64_t blocks = ((int64_t)M + (int64_t)R - 1) / (int64_t)R, waves = (blocks + m->sm_count - 1) / m->sm_count;
+    const double block = 2.0 * n + 0.02 * H + 1.75e-5 * (R + 0.3) * H * H + 1e-3 * n * H;
+    const double bit = 10.0 + (M < 64 ? 0.013 : 0.018) * H + (double)M * H * (3.5e-6 + 1.3e-9 * H);
+    return (double)waves * (waves > 1 ? 1.15 : 1.0) * block <= n * bit;
+}
+
 extern "C" lrs_status lrs_mlp_sample(lrs_mlp* m, int64_t count, uint64_t seed, int64_t sample0,
                                      uint64_t* y, float* logq, void* stream) {
     if (!m || count < 0 || (count > 0 && (!y || !logq))) return lrs_fail(LRS_ERR_ARG, "bad arguments");
@@ -1496,24 +1573,31 @@ extern "C" lrs_status lrs_mlp_sample(lrs_mlp* m, int64_t count, uint64_t seed, i
     cudaStream_t st = (cudaStream_t)stream;
     const int M = (int)count, H = m->H;
     lrs_status rc;
-    if ((rc = mlp_poll_err(m)) != LRS_OK) return rc;
-    // rows per block: eight, fewer where that leaves SMs without a block or the activations
-    // (8 H bytes a row) do not fit
-    auto launch = [&](auto kernel, int R) -> lrs_status {
-        const size_t smem = (size_t)R * H * 2 * sizeof(float);
+    if (sample_in_one(m, M)) {
+        if ((rc = mlp_poll_err(m)) != LRS_OK) return rc;
+        const int R = sample_rows(m, M);
+        const auto kernel = R == 8 ? k_sample<8> : R == 4 ? k_sample<4> : k_sample<2>;
         if (!lrs_capturing(st))
             LRS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMP_SMEM));
-        kernel<<<(unsigned)((M + R - 1) / R), SMP_TPB, smem, st>>>(m->b1, m->b2, m->b3, m->W1b, m->W2b, m->W3b, M, m->n, H,
-                                                                  m->NP, seed, sample0, y, logq);
+        kernel<<<(unsigned)((M + R - 1) / R), SMP_TPB, (size_t)R * H * 2 * sizeof(float), st>>>(
+            m->b1, m->b2, m->b3, m->W1b, m->W2b, m->W3b, M, m->n, H, m->NP, seed, sample0, y, logq);
         LRS_LAUNCH_CHECK("sample kernel");
+        mlp_post_err(m, st);
         return LRS_OK;
-    };
-    const int fit = SMP_SMEM / (H * 2 * (int)sizeof(float));
-    if (fit >= 8 && M > 608) rc = launch(k_sample<8>, 8);
-    else if (fit >= 4 && M > 304) rc = launch(k_sample<4>, 4);
-    else if (fit >= 2) rc = launch(k_sample<2>, 2);
-    else rc = lrs_fail(LRS_ERR_UNSUPPORTED, "hidden width %d too large for the sampler", H);
-    if (rc != LRS_OK) return rc;
+    }
+    const int Mp = pad64(count);
+    MlpWS w;
+    if ((rc = mlp_ws(m, Mp, w)) != LRS_OK) return rc;
+    if ((rc = mlp_poll_err(m)) != LRS_OK) return rc;
+    const int64_t tot = (int64_t)Mp * H;
+    k_sample_init<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(m->b1, Mp, H, M, w.Z1, w.H1, y, logq);
+    LRS_LAUNCH_CHECK("sample init");
+    for (int i = 0; i < m->n; ++i) {
+        if ((rc = gemm_tn(m, w.H1, H, m->W2b, H, Mp, H, H, EpiBiasReluBf16{m->b2, w.H2, H}, st)) != LRS_OK) return rc;
+        k_sample_bit<<<(unsigned)((M * 32 + 127) / 128), 128, 0, st>>>(w.H2, m->W3b, m->b3, m->W1b, M, H, m->NP,
+                                                                     i, seed, sample0, w.Z1, w.H1, y, logq);
+        LRS_LAUNCH_CHECK("sample bit");
+    }
     mlp_post_err(m, st);
     return LRS_OK;
 }
