@@ -562,7 +562,8 @@ lrs_status lrs_alu_probe(int32_t device, int64_t iters, double* ops_per_s);
  * per-term exact values.  The paper has no counterpart.
  *   LRS_TUNE_AMP_BLOCKS_PER_SM    amplitude grid target, blocks per SM (1..64, 8)
  *   LRS_TUNE_NORM_MAX_TILES       norm estimate, maximum term tiles (1..2^20, 2048)
- *   LRS_TUNE_MC_CHAINS_PER_BLOCK  Metropolis chains per block (1..64, 64)
+ *   LRS_TUNE_MC_CHAINS_PER_BLOCK  most Metropolis chains per block (1..64, 64; a block
+ *                                 takes no more than 32, whatever the value above)
  *   LRS_TUNE_NORM_MAX_FOLDS       norm estimate (-1..12, 12): accepted and returned;
  *                                 every term sums over y = G (s + x) restricted to the
  *                                 n - |v| constraints, on the route that its |v|

@@ -13,10 +13,13 @@ import os
 CANDIDATES = {
     "amp_blocks_per_sm": [2, 4, 8, 16, 32],
     "norm_max_tiles": [256, 512, 1024, 2048, 4096],
-    # fewer than 32 chains per block re-read each term's scalars (44 bytes) for too few
-    # chains; the knob itself accepts 1..64
+    # fewer than 32 chains per block re-read each term's coefficients for too few chains; a block
+    # takes 32 at most, so that 64 is the same launch
     "mc_chains_per_block": [32, 64],
-    "norm_max_folds": [-1, 4, 8, 12],
+    # changes nothing (include/lrstab.h): its default alone, since a search over a long norm
+    # estimate would choose between equal calls
+    "norm_max_folds": [12],
+    # changes nothing either; a search over 16 steps is short
     "mc_stages": [1, 2, 3, 4],
     "mc_lookahead": [1, 2],
 }

@@ -882,8 +882,7 @@ static lrs_status enqueue_steps(lrs_ctx* ctx, int64_t t0, int64_t count, float2*
 // pend, and may find the states and planes where they were).
 static lrs_status mc_graph(lrs_ctx* ctx, float2* partial, int32_t* jprop, cudaGraphExec_t* out) {
     const void* key[9] = {partial, jprop, ctx->Q, ctx->mc_planes, ctx->cx, ctx->cp, ctx->pend,
-                          (void*)(intptr_t)(((ctx->n_chains * 128 + ctx->tune_mc_cg) * 8 + ctx->tune_mc_stages) * 4 +
-                                            ctx->tune_mc_lookahead),
+                          (void*)(intptr_t)((ctx->n_chains * 128 + ctx->tune_mc_cg) * 4 + ctx->tune_mc_lookahead),
                           (void*)(intptr_t)ctx->cap};
     if (ctx->mc_exec && memcmp(key, ctx->mc_key, sizeof(key)) == 0) {
         *out = (cudaGraphExec_t)ctx->mc_exec;
