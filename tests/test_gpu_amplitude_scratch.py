@@ -93,3 +93,19 @@ def test_capture_after_a_call_of_the_other_kind(n):
         assert torch.equal(out, want)
         g.reset()
         sim.close()
+
+
+@pytest.mark.parametrize("n", [6, 7, 31, 33, 50, 62, 64])
+def test_blocks_of_several_tiles_equal_the_string_kernel(n):
+    """Few strings of many terms: blocks of 16, 8 or 4 string words and two to eight tiles."""
+    require_cuda()
+    for chi in (20000, 77824):
+        sim = _sim(n, chi)
+        for b in (3, 33, 100, 300):
+            x = _strings(sim, b)
+            want = torch.empty((b, 2), dtype=torch.float64, device="cuda")
+            sim.amplitude_noalloc(x, want)
+            err = torch.empty(b, dtype=torch.float32, device="cuda")
+            assert torch.equal(sim.amplitude(x), want), (chi, b)
+            assert torch.equal(sim.amplitude(x, err=err), want), (chi, b)
+        sim.close()
