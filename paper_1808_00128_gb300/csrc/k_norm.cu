@@ -67,17 +67,20 @@ __device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) {
 // The diagonal as two bit-planes (words 0 and 1 of the stream of l), the upper triangle
 // from words 2.. in the order (0,1), (0,2), .., (0,n-1), (1,2), .., one bit each.
 // One block per 32 states: lane l draws word j of its state, and 64 ballots turn the
-// 32 words into the bit-sliced entries 64 j .. 64 j + 63.
+// 32 words into the bit-sliced entries 64 j .. 64 j + 63.  States past L repeat state L - 1, and
+// their sums are dropped.  (As zero matrices they left sparse forms, whose isolated variables
+// sent the whole group through the elimination form by form: 16 states of the n = 57 QAOA at
+// chi = 2^17 9.4 ms, repeated 2.3.)
 constexpr int DRAW_WARPS = 8;
 __global__ void __launch_bounds__(32 * DRAW_WARPS) k_norm_draw(int n, int64_t L, uint64_t seed, NormPrep P) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t g = blockIdx.x, l = g * 32 + lane;
-    const uint64_t key = sm64_key(seed, (uint64_t)l);
+    const uint64_t key = sm64_key(seed, (uint64_t)(l < L ? l : L - 1));
     uint32_t* A = P.A + g * n * 64;
     const int entries = n * (n - 1) / 2;
     const int words = 2 + (entries + 63) / 64;
     for (int j = warp; j < words; j += DRAW_WARPS) {
-        const uint64_t w = l < L ? sm64_at(key, (uint64_t)j) : 0ull;
+        const uint64_t w = sm64_at(key, (uint64_t)j);
         uint32_t e0 = 0, e1 = 0;
 #pragma unroll
         for (int t = 0; t < 32; ++t) {
