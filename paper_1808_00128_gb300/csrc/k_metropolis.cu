@@ -85,22 +85,35 @@ __host__ __device__ __forceinline__ int mc_pairs(int n) { return n * (n - 1) / 2
 // of the constraints.
 constexpr int MC_PLANES = 4;
 
-__global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
+// A block takes a tile: its F in shared memory, and MC_SETS sets of 256 threads (a term each) that
+// share out the rows of J and the pairs of constraints, with the gridDim.y blocks of the tile where
+// there are fewer tiles than SMs.  (With one set, two warps a scheduler waited for one product
+// after the other: 130 us for four tiles at n = 57 and 520 us for 2^17 terms, now 17 and
+// 196.)  Padding terms have no weight and get no constraints: as |0^n> they have n of them,
+// which every chain would carry through the last tile.
+constexpr int MC_SETS = 4;
+__device__ __forceinline__ void mc_set_sync(int set) {
+    asm volatile("bar.sync %0, 256;" ::"r"(set + 1) : "memory");
+}
+
+__global__ void __launch_bounds__(256 * MC_SETS) k_mc_planes(TermsView T, McView V) {
     extern __shared__ uint64_t sF[];          // [n][256]
-    __shared__ uint32_t sw[2][64][16];        // words of a set of planes for the tile, double-buffered
+    __shared__ uint32_t sws[MC_SETS][2][64][16];   // words of a set of planes for the tile, double-buffered
     __shared__ int s_mf;
-    const int n = T.n, tid = threadIdx.x, lane = tid & 31, wi = tid >> 5;
+    const int n = T.n, set = threadIdx.x >> 8, tid = threadIdx.x & 255, lane = tid & 31, wi = tid >> 5;
+    const int first = blockIdx.y * MC_SETS + set, sets = gridDim.y * MC_SETS;   // of the tile's sets
     const int64_t tile = blockIdx.x, a = tile * MC_TERMS + tid;
     const int slot = (wi & 3) * 2 + (wi >> 2);   // word of this warp within the tile
-    for (int p = 0; p < n; ++p) sF[p * 256 + tid] = T.F[(int64_t)p * T.cap + a];
+    uint32_t(*sw)[64][16] = sws[set];
+    for (int p = set; p < n; p += MC_SETS) sF[p * 256 + tid] = T.F[(int64_t)p * T.cap + a];
     const uint64_t glo = T.glo[a], ghi = T.ghi[a], v = T.v[a], s = T.s[a];
     const uint32_t om = T.omega[a];
     const bool dead = ((om >> 3) & 1u) != 0u;
-    const uint64_t out = dead ? 0ull : ~v & T.nmask;
-    if (tid == 0) s_mf = 0;
+    const uint64_t out = dead || a >= T.chi ? 0ull : ~v & T.nmask;
+    if (threadIdx.x == 0) s_mf = 0;
     __syncthreads();
-    atomicMax(&s_mf, __popcll(out));
-    {
+    if (set == 0) atomicMax(&s_mf, __popcll(out));
+    if (first == 0) {
         float2 b = make_float2(0.f, 0.f);
         if (!dead) {
             b = z8_scale(T.coef[a], (int)(om & 7u), __popcll(v) + (int)(om >> 8));
@@ -108,10 +121,13 @@ __global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
         }
         V.base[(int64_t)((wi >> 2) * 32 + lane) * V.cols + tile * 4 + (wi & 3)] = b;
     }
+    __syncthreads();
+    const int mf = s_mf;
     const int64_t row = V.cols * 2;   // words per plane
     int buf = 0;
-    for (int p = 0; p < n; ++p, buf ^= 1) {
+    for (int p = first; p < n; p += sets, buf ^= 1) {
         const uint64_t Mp = T.M[(int64_t)p * T.cap + a], Fp = sF[p * 256 + tid];
+#pragma unroll 4
         for (int q = 0; q < p; ++q) {
             const uint32_t w = __ballot_sync(0xffffffffu, par64(Mp & sF[q * 256 + tid]));
             if (lane == 0) sw[buf][q][slot] = w;
@@ -123,21 +139,22 @@ __global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
             sw[buf][62][slot] = lo;
             sw[buf][63][slot] = hi;
         }
-        __syncthreads();
+        mc_set_sync(set);
         for (int e = tid; e < p * 8; e += 256)
             reinterpret_cast<uint32_t*>(V.J)[((int64_t)p * (p - 1) / 2 + (e >> 3)) * row + tile * 8 + (e & 7)] =
                 sw[buf][e >> 3][e & 7];
         if (tid < 16)
             reinterpret_cast<uint32_t*>(V.D)[(2 * p + (tid >> 3)) * row + tile * 8 + (tid & 7)] = sw[buf][62 + (tid >> 3)][tid & 7];
     }
-    const int mf = s_mf;
     uint64_t ks = out;
     const int slot4 = (wi & 3) * 4 + (wi >> 2);   // word of this warp in a set of pairs
-    for (int i = 0; 2 * i < mf; ++i, buf ^= 1) {
+    for (int i = 0; 2 * i < mf; ++i) {
         const int k0 = ks ? ffs64(ks) : -1;   // constraint 2 i of this term: qubit k0, or none
         ks &= ks - 1;
         const int k1 = ks ? ffs64(ks) : -1;
         ks &= ks - 1;
+        if (i % sets != first) continue;
+#pragma unroll 4
         for (int p = 0; p <= n; ++p) {
             const uint64_t r = p < n ? sF[p * 256 + tid] : s;   // last: the targets
             const uint32_t w0 = __ballot_sync(0xffffffffu, k0 >= 0 ? (uint32_t)getb(r, k0) : 0u);
@@ -147,15 +164,17 @@ __global__ void __launch_bounds__(256) k_mc_planes(TermsView T, McView V) {
                 sw[buf][p][slot4 + 2] = w1;
             }
         }
-        __syncthreads();
+        mc_set_sync(set);
         for (int e = tid; e < (n + 1) * 16; e += 256) {
             const int p = e >> 4;
             uint4* dst = p < n ? V.K + ((int64_t)p * V.pairs + i) * V.cols : V.target + (int64_t)i * V.cols;
             reinterpret_cast<uint32_t*>(dst)[tile * 16 + (e & 15)] = sw[buf][p][e & 15];
         }
+        buf ^= 1;
     }
-    if (tid == 0) V.mf[tile] = (uint8_t)mf;
-    if (tid < 8) reinterpret_cast<uint32_t*>(V.J)[mc_pairs(n) * row + tile * 8 + tid] = 0u;
+    if (blockIdx.y > 0) return;
+    if (threadIdx.x == 0) V.mf[tile] = (uint8_t)mf;
+    if (threadIdx.x < 8) reinterpret_cast<uint32_t*>(V.J)[mc_pairs(n) * row + tile * 8 + threadIdx.x] = 0u;
 }
 
 __device__ __forceinline__ uint2 operator^(uint2 a, uint2 b) { return make_uint2(a.x ^ b.x, a.y ^ b.y); }
@@ -178,21 +197,29 @@ __device__ __forceinline__ int mc_row(int p, int q, int zero) {
     return p == q ? zero : hi * (hi - 1) / 2 + lo;
 }
 
-// State of every (chain, term) at the chains' strings: q(x) by adding the set bits in order,
-// and the syndromes.
+// State of every (chain, term) at the chains' strings: q(x) by adding the set bits (Z4 sums, so in
+// any order), and the syndromes.  `split` threads of a warp (a power of two, their columns tbx = 32
+// / split apart) share the set bits and the pairs of constraints of a (chain, column): with
+// few chains of few terms one thread's loads, one batch after the other, were all there was to wait
+// for (8 chains of 1000 terms at n = 57: 121 us, now 29).
 __global__ void __launch_bounds__(MC_TPB) k_mc_start(McView V, int64_t C, uint2* __restrict__ S,
-                                                     const uint64_t* __restrict__ xs, uint64_t nmask, int tbx,
+                                                     const uint64_t* __restrict__ xs, uint64_t nmask, int tbx, int split,
                                                      int64_t cblocks) {
     // chains fastest: the blocks that read one column range's planes run together
-    const int tid = threadIdx.x;
-    const int64_t tb = blockIdx.x / cblocks, c = blockIdx.x % cblocks * (MC_TPB / tbx) + tid / tbx;
-    const int64_t col = tb * tbx + tid % tbx;
-    if (c >= C || col >= V.cols) return;
+    const int tid = threadIdx.x, part = tid / tbx % split;
+    int64_t c = blockIdx.x % cblocks * (MC_TPB / (tbx * split)) + tid / (tbx * split);
+    int64_t col = blockIdx.x / cblocks * tbx + tid % tbx;
+    const bool on = c < C && col < V.cols;
+    if (split == 1 && !on) return;
+    if (!on) c = col = 0;   // for the exchanges
     const uint64_t x = xs[c] & nmask;
     const uint2* J = V.J + col;
     uint2 lo = make_uint2(0u, 0u), hi = lo;
-    for (uint64_t r = x; r; r &= r - 1) {
+    uint64_t r = x;
+    for (int k = 0; k < part; ++k) r &= r - 1;
+    while (r) {
         const int p = ffs64(r);
+        for (int k = 0; k < split; ++k) r &= r - 1;
         uint2 par = make_uint2(0u, 0u);
         const uint2* Jp = J + (int64_t)(p * (p - 1) / 2) * V.cols;
         uint64_t below = x & (bit64(p) - 1);
@@ -209,23 +236,35 @@ __global__ void __launch_bounds__(MC_TPB) k_mc_start(McView V, int64_t C, uint2*
         z4_step(lo, hi, __ldg(V.D + (int64_t)(2 * p) * V.cols + col), __ldg(V.D + (int64_t)(2 * p + 1) * V.cols + col), false,
                 par);
     }
+    for (int off = tbx; off < tbx * split; off <<= 1) {
+        uint2 l2, h2;
+        l2.x = __shfl_xor_sync(0xffffffffu, lo.x, off);
+        l2.y = __shfl_xor_sync(0xffffffffu, lo.y, off);
+        h2.x = __shfl_xor_sync(0xffffffffu, hi.x, off);
+        h2.y = __shfl_xor_sync(0xffffffffu, hi.y, off);
+        hi = hi ^ h2 ^ (lo & l2);
+        lo = lo ^ l2;
+    }
+    if (!on) return;
     const int64_t plane = C * V.cols;
     uint2* st = S + c * V.cols + col;
-    st[0] = lo;
-    st[plane] = hi;
+    if (part == 0) {
+        st[0] = lo;
+        st[plane] = hi;
+    }
     uint4* sy = reinterpret_cast<uint4*>(S + MC_PLANES * plane) + c * V.cols + col;
     const int pairs = (V.mf[col >> 2] + 1) >> 1;
-    for (int i = 0; i < pairs; ++i) {
+    for (int i = part; i < pairs; i += split) {
         uint4 y = __ldg(V.target + (int64_t)i * V.cols + col);
         const uint4* Ki = V.K + (int64_t)i * V.cols + col;
-        uint64_t r = x;
-        while (r) {
+        uint64_t w = x;
+        while (w) {
             uint4 t[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 t[u] = make_uint4(0u, 0u, 0u, 0u);
-                if (r) t[u] = __ldg(Ki + (int64_t)ffs64(r) * V.pairs * V.cols);
-                r &= r - 1;
+                if (w) t[u] = __ldg(Ki + (int64_t)ffs64(w) * V.pairs * V.cols);
+                w &= w - 1;
             }
             y = y ^ (t[0] ^ t[1]) ^ (t[2] ^ t[3]);
         }
@@ -293,7 +332,10 @@ __global__ void __launch_bounds__(MC_TPB, 3) k_mc_pass(McView V, int64_t C, uint
             extra = 16;
         }
         mc_bar_expect(bar, (uint32_t)(64 * nb * sizeof(float2)) + extra);
-        for (int r = 0; r < 64; ++r)
+    }
+    if (tid < 32) {
+        __syncwarp();
+        for (int r = tid; r < 64; r += 32)
             mc_bulk_load(mc_smem(sbase + r * tbx), V.base + (int64_t)r * V.cols + col0, (uint32_t)(nb * sizeof(float2)), bar);
     }
     for (int ci = tid >> 5; ci < nc; ci += MC_TPB / 32) {   // a warp per chain
@@ -785,10 +827,13 @@ static lrs_status mc_start(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) {
     if (!ctx->mc_direct) {
         McView V;
         mc_layout(ctx, &V);
-        const int tbx = mc_columns(V.cols), nsub = MC_TPB / tbx;
+        // as many threads a (chain, column) as leave no more than two rounds of 2048 an SM
+        int split = 8;
+        while (split > 1 && C * V.cols * split > (int64_t)4096 * ctx->sm_count) split /= 2;
+        const int tbx = split > 1 ? 32 / split : mc_columns(V.cols), nsub = MC_TPB / (tbx * split);
         const int64_t cblocks = (C + nsub - 1) / nsub, blocks = (V.cols + tbx - 1) / tbx * cblocks;
         if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "chain start grid too large");
-        k_mc_start<<<(unsigned)blocks, MC_TPB, 0, st>>>(V, C, (uint2*)ctx->Q, x, ctx->nmask, tbx, cblocks);
+        k_mc_start<<<(unsigned)blocks, MC_TPB, 0, st>>>(V, C, (uint2*)ctx->Q, x, ctx->nmask, tbx, split, cblocks);
         LRS_LAUNCH_CHECK("chain start kernel");
     }
     double* amp = nullptr;
@@ -808,7 +853,10 @@ lrs_status launch_chains_init(lrs_ctx* ctx, const uint64_t* x, cudaStream_t st) 
     if (!lrs_capturing(st))
         LRS_CUDA(cudaFuncSetAttribute(k_mc_planes, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)(62 * 256 * sizeof(uint64_t))));
-    k_mc_planes<<<(unsigned)(ctx->cap / MC_TERMS), 256, smem, st>>>(ctx->view(), V);
+    const int64_t tiles = ctx->cap / MC_TERMS;
+    int parts = 8;
+    while (parts > 1 && tiles * parts > ctx->sm_count) parts /= 2;
+    k_mc_planes<<<dim3((unsigned)tiles, (unsigned)parts), 256 * MC_SETS, smem, st>>>(ctx->view(), V);
     LRS_LAUNCH_CHECK("chain planes kernel");
     return mc_start(ctx, x, st);
 }
@@ -831,12 +879,9 @@ static lrs_status mc_pass(lrs_ctx* ctx, int steps, const int32_t* jprop, float2*
     const int64_t groups = (C + cg - 1) / cg, blocks = tblocks * groups;
     if (blocks > 0x7FFFFFFF) return lrs_fail(LRS_ERR_UNSUPPORTED, "Metropolis grid too large");
     const size_t smem = (size_t)64 * tbx * sizeof(float2) + cg * sizeof(McChain);
-    if (steps == 2)
-        k_mc_pass<2><<<(unsigned)blocks, MC_TPB, smem, st>>>(V, C, (uint2*)ctx->Q, ctx->cx, ctx->pend, jprop, partial,
-                                                             (int)cg, groups, tbx, ctx->mc_err_d);
-    else
-        k_mc_pass<1><<<(unsigned)blocks, MC_TPB, smem, st>>>(V, C, (uint2*)ctx->Q, ctx->cx, ctx->pend, jprop, partial,
-                                                             (int)cg, groups, tbx, ctx->mc_err_d);
+    const auto kernel = steps == 2 ? k_mc_pass<2> : k_mc_pass<1>;
+    kernel<<<(unsigned)blocks, MC_TPB, smem, st>>>(V, C, (uint2*)ctx->Q, ctx->cx, ctx->pend, jprop, partial, (int)cg,
+                                                   groups, tbx, ctx->mc_err_d);
     LRS_LAUNCH_CHECK("metropolis pass kernel");
     return LRS_OK;
 }
@@ -860,7 +905,9 @@ static lrs_status enqueue_steps(lrs_ctx* ctx, int64_t t0, int64_t count, float2*
     if (ctx->tune_mc_lookahead == 2) {
         for (; t + 1 < t0 + count; t += 2) {
             if ((rc = mc_pass(ctx, 2, jprop, partial, st)) != LRS_OK) return rc;
-            k_metro_accept2<<<(unsigned)C, n_tiles >= 1024 ? 768 : 256, 0, st>>>(partial, n_tiles, ctx->mc_par, t, ctx->n, ctx->cx,
+            // three groups where the sums are long, or where there are too few chains to fill the GPU
+            const int tpb = n_tiles >= 1024 || C <= 2 * ctx->sm_count ? 768 : 256;
+            k_metro_accept2<<<(unsigned)C, tpb, 0, st>>>(partial, n_tiles, ctx->mc_par, t, ctx->n, ctx->cx,
                                                           ctx->cp, ctx->pend, jprop,
                                                           trace ? trace + t * C : nullptr, C);
             LRS_LAUNCH_CHECK("metropolis two-step accept kernel");
