@@ -524,6 +524,15 @@ class StepRunner:
             self._look = self.sim.get_tuning("mc_lookahead")
         return self._look
 
+    @property
+    def amp_grid(self):
+        """SMs and amplitude blocks per SM (read while the context is open and kept)."""
+        if getattr(self, "_grid", None) is None:
+            import torch
+            self._grid = (torch.cuda.get_device_properties(self.dev).multi_processor_count,
+                          self.sim.get_tuning("amp_blocks_per_sm"))
+        return self._grid
+
     def step(self, ev=None, idx=0):
         st = self.stream
 
@@ -600,12 +609,9 @@ class StepRunner:
     def launches(self):
         """Library kernels one step launches."""
         s = self.shape
-        if getattr(self, "_bps", None) is None:
-            import torch
-            self._bps = (torch.cuda.get_device_properties(self.dev).multi_processor_count,
-                         self.sim.get_tuning("amp_blocks_per_sm"))
-        return (launches_per_step(s["T"], self.lookahead) + record_launches(self.n, self.chi, s["B"], 1024, *self._bps) - 1
-                + 2 + record_launches(self.n, self.chi, s["C"], 512, *self._bps) - 1)
+        grid = self.amp_grid
+        return (launches_per_step(s["T"], self.lookahead) + record_launches(self.n, self.chi, s["B"], 1024, *grid) - 1
+                + 2 + record_launches(self.n, self.chi, s["C"], 512, *grid) - 1)
 
     def rooflines(self, phase_ms, alu_peak, hbm_peak):
         """Per phase: achieved and fraction of the roofline on the kernel's own op count
@@ -662,6 +668,7 @@ class StepRunner:
 
     def close(self):
         _ = self.lookahead          # kept for the launch count after the context is gone
+        self.lookahead, self.amp_grid   # what launches() needs of the context
         self.sim.close()
 
 

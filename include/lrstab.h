@@ -286,9 +286,11 @@ lrs_status lrs_amplitude(lrs_ctx* ctx, const uint64_t* x_dev, int64_t batch, dou
                          float* err_est_dev, void* stream);
 
 /* lrs_amplitude for several circuits (contexts with the same qubit count on one
- * device, e.g. decompositions of uneven chi) in two launches: one amplitude launch
- * covering every circuit's term tiles (at most 12 circuits per launch; more take
- * further launches) and one FP64 reduction for all their strings.  Circuit i gets
+ * device, e.g. decompositions of uneven chi).  Small ones (on average less than 2^23
+ * (x, term) pairs a circuit) share two launches: one amplitude launch covering every
+ * circuit's term tiles (at most 12 circuits per launch; more take further launches)
+ * and one FP64 reduction for all their strings.  Larger ones, each of which fills the
+ * GPU, run one after the other as lrs_amplitude would.  Circuit i gets
  * batch[i] strings x_dev[i] and writes out_dev[i] (2 batch[i] doubles), with the tile
  * plan of its own lrs_amplitude call, so its values equal that call's bit for bit.
  * Errors: LRS_ERR_ARG (NULL or repeated contexts, different devices or widths),

@@ -554,8 +554,8 @@ def metropolis_learned(sim: "Simulator", mlp: MLP, steps: int, seed: int, step0:
 
 
 def amplitude_batch(sims, xs, outs=None, stream=None):
-    """lrs_amplitude_batch: <x|psi> of several circuits (same width, one device) in one
-    amplitude launch and one reduction; returns float64 CUDA tensors [B_i, 2]."""
+    """lrs_amplitude_batch: <x|psi> of several circuits (same width, one device), small ones in
+    shared launches, large ones one after the other; returns float64 CUDA tensors [B_i, 2]."""
     import torch
     k = len(sims)
     if outs is None:
