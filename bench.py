@@ -667,8 +667,7 @@ class StepRunner:
                 "norm_estimate": norm ** 2, "relative_to": "max(|a|, ||psi|| 2^{-n/2})"}
 
     def close(self):
-        _ = self.lookahead          # kept for the launch count after the context is gone
-        self.lookahead, self.amp_grid   # what launches() needs of the context
+        _ = self.lookahead, self.amp_grid   # kept for the launch count after the context is gone
         self.sim.close()
 
 
@@ -1331,7 +1330,7 @@ def hidden_shift_sum8_chain_study(local=0, chi=1 << 24, flip_steps=32, learned_s
         return float(np.max(np.abs(pc - pa) / np.maximum(pa, 1e-30)))
 
     out = {"workload": f"hidden_shift_n40_ccz16_sum8_chi{chi}", "chi": chi, "chains": C,
-           "pauli_state_gb": C * chi * 12 / 1e9, "chains_started_at_s": start_at_s}
+           "state_gb_at_most": C * chi * (4 + (n + 1) // 2 * 2) / 8 / 1e9, "chains_started_at_s": start_at_s}
     xo = torch.empty(C, dtype=torch.int64, device=dev)
     po = torch.empty(C, dtype=torch.float64, device=dev)
     # (a) chains at s

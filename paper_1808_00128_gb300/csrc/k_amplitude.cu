@@ -356,6 +356,13 @@ __global__ void __launch_bounds__(256) k_amp_prep(TermsView T, AmpPrep P) {
     if (r >= P.tt || a >= T.cap) return;
     const uint64_t v = T.v[a], s = T.s[a], glo = T.glo[a], ghi = T.ghi[a];
     const uint32_t om = T.omega[a];
+    uint64_t F[2], M[2], J[2] = {0, 0};   // on their way before the flags are known
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int q = lane + 32 * c;
+        F[c] = q < n ? T.F[(int64_t)q * T.cap + a] : 0ull;
+        M[c] = q < n ? T.M[(int64_t)q * T.cap + a] : 0ull;
+    }
     uint64_t* rec = P.rec + ((int64_t)blockIdx.y * P.rl + j) * P.words;
     const bool live = ((om >> 3) & 1u) == 0u;
     const uint64_t out = ~v & T.nmask;
@@ -369,13 +376,10 @@ __global__ void __launch_bounds__(256) k_amp_prep(TermsView T, AmpPrep P) {
         rec[AMP_VAL] = (uint64_t)__float_as_uint(val.x) | (uint64_t)__float_as_uint(val.y) << 32;
     }
     if (!live) return;
-    uint64_t F[2], M[2], J[2] = {0, 0};
     uint32_t hi[2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
         const int q = lane + 32 * c;
-        F[c] = q < n ? T.F[(int64_t)q * T.cap + a] : 0ull;
-        M[c] = q < n ? T.M[(int64_t)q * T.cap + a] : 0ull;
         hi[c] = (uint32_t)getb(ghi, q) ^ par64(F[c] & M[c]) ^ par64(F[c] & s & v);
     }
     uint64_t* rows = sF[threadIdx.x >> 5];
