@@ -250,10 +250,10 @@ def launches_per_step(T, lookahead=1):
 # dram__bytes_write.sum), per unit of work, with the hash of the kernel source the
 # capture ran; `traffic` is reported only while that source is unchanged.
 TRAFFIC = {
-    # k_norm<52, 0> on the profiling case (n = 50 QAOA, chi = 2^16, L = 64): 35,185,664 B
-    # read + 2,357,760 B written per launch for 2^16 x 64 (A, term) units
-    "norm_estimate": {"bytes_per_unit": (35185664 + 2357760) / (65536 * 64),
-                      "source": "paper_1808_00128_gb300/csrc/k_norm.cu", "sha16": "409e8ed765041395",
+    # k_norm<52, 0> on the profiling case (n = 50 QAOA, chi = 2^16, L = 64): 33,972,992 B
+    # read + 2,328,576 B written per launch for 2^16 x 64 (A, term) units
+    "norm_estimate": {"bytes_per_unit": (33972992 + 2328576) / (65536 * 64),
+                      "source": "paper_1808_00128_gb300/csrc/k_norm.cu", "sha16": "cc7180035a246d39",
                       "profile": "profiles/k_norm_n50_chi65536_L64.md"},
 }
 

@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(MC_TPB) k_mc_start(McView V, int64_t C, uint2*
 // The FP32 sums are what bounds it: per (term, sum) a sign and live factor (+-2 or +-0, built
 // from two adjacent bits of a nibble and multiplied onto half the coefficient, which is
 // exact), a swap of the two parts, and one fused multiply-add each.
-// n = 50, chi = 2^20, 256 chains: 520 us per two-step pass and about 20 for its accept test
+// n = 50, chi = 2^20, 256 chains: 574 us per two-step pass and 37 for its accept test
 // (2.1 ms with 16-byte Pauli states); n = 40, chi = 2^16, 1024 chains: 136 us.
 // The block's coefficients (64 rows of tbx columns) are copied once by cp.async.bulk; the wait
 // is bounded (1 s) and a block that gives up sets *err and leaves its sums unwritten.
